@@ -265,6 +265,14 @@ __host__ __device__ inline Lay make_lay(int N, int nu, int threads) {
   return L;
 }
 
+// Shared-memory elements of the plain form's kernels: PIPG runs T threads, the
+// others Tr, and the discretization's stage buffers grow with the threads, so
+// that on short grids the layout for Tr > T is the larger one.
+__host__ __device__ inline int plain_total(int N, int nu, int T, int Tr) {
+  const int a = make_lay(N, nu, T).total, b = make_lay(N, nu, Tr).total;
+  return a > b ? a : b;
+}
+
 // ---------------------------------------------------------------------------
 // block reductions (every thread of the CTA must call them)
 // ---------------------------------------------------------------------------

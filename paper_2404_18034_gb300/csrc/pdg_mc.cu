@@ -1038,7 +1038,7 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T;
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)L.total * sizeof(R);
+  const size_t smem = (size_t)(mode == 0 ? plain_total(h->n_max, NU, T, pl.Tr) : L.total) * sizeof(R);
   if (L.ipw < 1 || make_lay(h->n_max, NU, pl.Tr).ipw < 1)
     return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
   if (int rc = Kern<R, NU>::prepare(h, T, smem)) return rc;
@@ -1231,7 +1231,7 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.pv);
   h->last_variant = pl.pv;
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)L.total * sizeof(R);
+  const size_t smem = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
   if (int rc = Kern<R, NU>::prepare(h, T, smem)) return rc;
   const size_t istride = (size_t)L.img;
   const size_t need = istride * sizeof(R) * B;
@@ -1307,7 +1307,7 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   const int T = pl.T, Tr = pl.Tr;
   const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.pv);
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)L.total * sizeof(R);
+  const size_t smem = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
   if (L.ipw < 1) return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t istride = (size_t)L.img;
