@@ -388,7 +388,10 @@ k_plain_pipg(const DParams P, int B, int Nmax, const int* __restrict__ Ns, Plain
   const int N = Ns ? Ns[b] : Nmax;
   const Lay L = make_lay(N, NU, blockDim.x);
   R* img = reinterpret_cast<R*>(W.img) + (size_t)b * W.istride;
-  copy_g2s(sm + L.Am, img + L.Am, L.img - L.Am);     // subproblem + warm start
+  // subproblem + warm start; the thrust projection also reads the reference
+  // controls, which lie right before the subproblem
+  const int from = P.soc ? L.Ub : L.Am;
+  copy_g2s(sm + from, img + from, L.img - from);
   __syncthreads();
   const R sigma = img[L.sc + 0];
   const int it = run_pipg<R, NU, PV>(P, L, sm, sigma, force ? force[2 * b + 1] : 0);
