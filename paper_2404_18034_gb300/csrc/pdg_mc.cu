@@ -70,20 +70,34 @@ using namespace pdg;
 #ifndef PDG_KS_PERS_MAXT
 #define PDG_KS_PERS_MAXT 512
 #endif
+// The fixed-point loop of FP64 instances (internal variant 4): at most 256
+// threads (N = 32), so up to 255 registers for its tiles.
+#define PDG_FX_MAXT 256
 #define PDG_LB_PERS(R, PV)                                                                  \
-  __launch_bounds__((PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT                            \
+  __launch_bounds__((PV) == 4 ? PDG_FX_MAXT : (PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT  \
                     : ((PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512)), \
                     sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 #define PDG_LB(R, PV)                                                                       \
-  __launch_bounds__((PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512), \
+  __launch_bounds__((PV) == 4 ? PDG_FX_MAXT                                                   \
+                    : (PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512), \
                     sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 
 namespace {
 
+// The FP64 loop behind the fixed-point one, out of line: it runs where the
+// data does not suit 64-bit fixed point.
+template <int NU>
+__device__ __noinline__ int pipg_fp64(const DParams& P, const Lay& L, double* sm, double sigma, int force) {
+  return phase_pipg<double, NU>(P, L, sm, sigma, force);
+}
+
 template <typename R, int NU, int PV, bool CK = false>
 __device__ __forceinline__ int run_pipg(const DParams& P, const Lay& L, R* sm, R sigma, int force,
                                         double* ck = nullptr) {
-  if constexpr (PV == 2) return phase_pipg_reg<R, NU>(P, L, sm, sigma, force);
+  if constexpr (PV == 4) {
+    const int it = phase_pipg_fx<NU>(P, L, sigma, force);
+    return it >= 0 ? it : pipg_fp64<NU>(P, L, sm, sigma, force);
+  } else if constexpr (PV == 2) return phase_pipg_reg<R, NU>(P, L, sm, sigma, force);
   else if constexpr (PV == 3) return phase_pipg_ks<R, NU>(P, L, sm, sigma, force);
   else return phase_pipg<R, NU, CK>(P, L, sm, sigma, force, ck);
 }
@@ -963,7 +977,15 @@ struct Plan {
   int T;   // threads of the solve kernel (and of k_plain_pipg)
   int Tr;  // threads of the other plain-form kernels
   int pv;  // 1 shared-memory PIPG, 2 register PIPG, 3 register tiles
+  int kv;  // the kernels' PIPG loop: pv, or 4 where form 1 runs in fixed point
 };
+
+// Shared memory of a solve kernel for instances of up to N nodes with T threads.
+template <typename R>
+static size_t solve_smem(int N, int nu, int T, int kv) {
+  const Lay L = make_lay(N, nu, T);
+  return (size_t)(kv == 4 ? make_fx_lay(L).end : L.total) * sizeof(R);
+}
 
 static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bool use_override = true) {
   const int treg = pipg_reg_threads(N, h->p.nu);
@@ -979,7 +1001,7 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
              " threads per CTA at N = " + std::to_string(N);
       return false;
     }
-    *out = {T, T < 512 ? T : 512, 2};
+    *out = {T, T < 512 ? T : 512, 2, 2};
   } else if (pv == 3) {
     // the lane groups' threads, at least two warps (the discretization wants
     // one interval per wave); the plain form's other kernels at least 128
@@ -990,11 +1012,19 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
              " threads per CTA at N = " + std::to_string(N);
       return false;
     }
-    *out = {T, T < 128 ? 128 : T, 3};
+    *out = {T, T < 128 ? 128 : T, 3, 3};
   } else {
-    const int T = ov > 0 ? ov : threads_for(N, h->p.nu, h->p.precision);
+    // FP64 runs the loop in 64-bit fixed point (phase_pipg_fx: 5 to 8 times
+    // the FP64 loop's rate at every N) wherever its lane groups and its
+    // exchange region fit; not with the thrust projection, whose square roots
+    // are FP64 work, nor in the gradient's solve, which records FP64 states
+    int T = ov > 0 ? ov : threads_for(N, h->p.nu, h->p.precision);
     if (T > 512) { *why = "the shared-memory PIPG form runs at most 512 threads per CTA"; return false; }
-    *out = {T, T, 1};
+    bool fx = h->p.precision == 0 && !h->p.soc_thrust && !h->ck_rec;
+    if (fx && ov == 0) T = T < tks ? tks : (T > PDG_FX_MAXT ? PDG_FX_MAXT : T);
+    fx = fx && T >= tks && T <= PDG_FX_MAXT && solve_smem<double>(N, h->p.nu, T, 4) <= 226 * 1024;
+    if (!fx && ov == 0) T = threads_for(N, h->p.nu, h->p.precision);
+    *out = {T, T, 1, fx ? 4 : 1};
   }
   return true;
 }
@@ -1009,10 +1039,16 @@ static PersistentFn<R, NU> persistent_fn(int pv, bool ck = false) {
   if constexpr (sizeof(R) == 8) {
     if (ck && pv == 1) return k_persistent<R, NU, 1, true>;
   }
+  if constexpr (sizeof(R) == 8) {
+    if (pv == 4) return k_persistent<R, NU, 4>;
+  }
   return pv == 3 ? k_persistent<R, NU, 3> : (pv == 2 ? k_persistent<R, NU, 2> : k_persistent<R, NU, 1>);
 }
 template <typename R, int NU>
 static PlainPipgFn<R, NU> plain_pipg_fn(int pv) {
+  if constexpr (sizeof(R) == 8) {
+    if (pv == 4) return k_plain_pipg<R, NU, 4>;
+  }
   return pv == 3 ? k_plain_pipg<R, NU, 3> : (pv == 2 ? k_plain_pipg<R, NU, 2> : k_plain_pipg<R, NU, 1>);
 }
 
@@ -1026,9 +1062,11 @@ struct Kern {
                          (const void*)k_plain_pipg<R, NU, 3>, (const void*)k_plain_update<R, NU>,
                          (const void*)k_subproblem<R, NU>};
     for (const void* f : fns) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if constexpr (sizeof(R) == 8)
-      PDG_CUDA(h, cudaFuncSetAttribute(k_persistent<R, NU, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
+    if constexpr (sizeof(R) == 8) {
+      const void* fp64[] = {(const void*)k_persistent<R, NU, 1, true>, (const void*)k_persistent<R, NU, 4>,
+                            (const void*)k_plain_pipg<R, NU, 4>};
+      for (const void* f : fp64) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    }
     return 0;
   }
 };
@@ -1041,11 +1079,13 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T;
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)(mode == 0 ? plain_total(h->n_max, NU, T, pl.Tr) : L.total) * sizeof(R);
+  // of the persistent kernel or the plain form's PIPG kernel, and of the plain form's others
+  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, pl.Tr) * sizeof(R);
   if (L.ipw < 1 || make_lay(h->n_max, NU, pl.Tr).ipw < 1)
     return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
-  if (int rc = Kern<R, NU>::prepare(h, T, smem)) return rc;
-  const PersistentFn<R, NU> kp = persistent_fn<R, NU>(pl.pv, h->ck_rec && mode == 1);
+  if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
+  const PersistentFn<R, NU> kp = persistent_fn<R, NU>(pl.kv, h->ck_rec && mode == 1);
   int occ = 0;
   PDG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, T, smem));
   if (occ < 1) return fail(h, PDG_EINVAL, "solve kernel does not fit on an SM with this configuration");
@@ -1093,9 +1133,9 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
       Plan pn;
       if (!plan_for(h, N, &pn, &why, N == h->n_max)) return fail(h, PDG_EINVAL, why);
       const int Tn = pn.T;
-      const PersistentFn<R, NU> kpn = persistent_fn<R, NU>(pn.pv);
+      const PersistentFn<R, NU> kpn = persistent_fn<R, NU>(pn.kv);
       const Lay Ln = make_lay(N, NU, Tn);
-      const size_t smem_n = (size_t)Ln.total * sizeof(R);
+      const size_t smem_n = solve_smem<R>(N, NU, Tn, pn.kv);
       if (Ln.ipw < 1) continue;
       int occ_n = 0;
       PDG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_n, kpn, Tn, smem_n));
@@ -1155,15 +1195,15 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   W.lit = h->lit;
   PDG_CUDA(h, cudaMemsetAsync(W.done, 0, sizeof(int), s));
   const int Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.pv);
-  k_plain_init<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
+  k_plain_init<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
   PDG_CUDA(h, cudaGetLastError());
   cudaGraph_t graph = nullptr;
   PDG_CUDA(h, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  k_plain_disc<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W);
-  k_plain_power<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
+  k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+  k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
   kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
-  k_plain_update<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters, pipg_iters,
+  k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters, pipg_iters,
                                              trace, nullptr);
   cudaError_t ce = cudaStreamEndCapture(s, &graph);
   if (ce != cudaSuccess) return fail(h, PDG_ECUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
@@ -1231,11 +1271,12 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   std::string why;
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.pv);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
   h->last_variant = pl.pv;
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
-  if (int rc = Kern<R, NU>::prepare(h, T, smem)) return rc;
+  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
+  if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
   const size_t istride = (size_t)L.img;
   const size_t need = istride * sizeof(R) * B;
   if (h->img_bytes < need) {
@@ -1270,10 +1311,10 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   W.done = h->ints + 4 * (size_t)B;
   W.lit = h->lit;
   k_pack<R, NU><<<B, 128, 0, s>>>(B, h->n_max, T, x0, Ns, W, 0, X, U, xh, uh, mup, mum, phi, th, sigma, defect, iters);
-  k_plain_disc<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W);
-  k_plain_power<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, force);
+  k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+  k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, force);
   kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, force);
-  k_plain_update<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, 1, nullptr, nullptr, nullptr, nullptr, nullptr,
+  k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 1, nullptr, nullptr, nullptr, nullptr, nullptr,
                                              nullptr, nullptr, nullptr, step);
   k_pack<R, NU><<<B, 128, 0, s>>>(B, h->n_max, T, x0, Ns, W, 1, X, U, xh, uh, mup, mum, phi, th, sigma, defect, iters);
   PDG_CUDA(h, cudaGetLastError());
@@ -1308,9 +1349,10 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   std::string why;
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.pv);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
+  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
   if (L.ipw < 1) return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t istride = (size_t)L.img;
@@ -1326,7 +1368,7 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   }
   void* base = nullptr;
   if (int rc = noalloc_scratch(h, &base)) return rc;
-  if (int rc = Kern<R, NU>::prepare(h, T, smem)) return rc;
+  if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
   char* c = (char*)base;
   PlainWs W;
   W.st = (int*)c;
@@ -1342,12 +1384,12 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   // the array keeps the previous call's contents: clear the counter (every
   // per-instance field is written by k_plain_init before it is read)
   PDG_CUDA(h, cudaMemsetAsync(W.done, 0, sizeof(int), s));
-  k_plain_init<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
+  k_plain_init<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
   for (int j = 0; j < h->p.scp_jmax; ++j) {
-    k_plain_disc<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W);
-    k_plain_power<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
+    k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+    k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
     kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
-    k_plain_update<R, NU><<<B, Tr, smem, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters,
+    k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters,
                                                pipg_iters, nullptr, nullptr);
   }
   PDG_CUDA(h, cudaGetLastError());

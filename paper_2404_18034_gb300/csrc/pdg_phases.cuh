@@ -1469,6 +1469,10 @@ __device__ PDG_PKS_ATTR int phase_pipg_ks(const DParams& P, const Lay& L, R* /*i
   return j;
 }
 
+}  // namespace pdg
+#include "pdg_pipg_fx.cuh"
+namespace pdg {
+
 // SCP update (Sec. 2.3.2: x = P_x x_hat + xbar) and convergence test
 // (reading: scaled step, scaled defect and CTCS budget).  Returns the scaled
 // step; *nonfinite is set when X or U holds a non-finite value.

@@ -1,0 +1,642 @@
+// pdg_pipg_fx.cuh -- PIPG_custom of an FP64 instance in 64-bit fixed point.
+#pragma once
+
+namespace pdg {
+
+// ---------------------------------------------------------------------------
+// Why integers.  GB300 issues two FP64 FMAs a clock and SM, and 64 of the
+// 32 x 32 + 64-bit integer multiply-adds (measured: 0.052 and 1.93 warp
+// instructions a clock and SM), so the FP64 loop of phase_pipg is bound by
+// the FP64 pipe, where three integer multiply-adds in place of one FMA cost a
+// twelfth.  This loop has no floating-point instruction in it.
+//
+// Variables.  With psi = phi / sqrt(omega), theta likewise, gamma = alpha
+// sqrt(omega) and M = gamma K, the iteration of Alg. PIPG_custom reads
+//   x' = c1 x~ - M^T psi~ + ...,  psi' = psi~ + M (2 x' - x~) + gamma (w + ...)
+// so one matrix M of spectral norm at most one serves both steps, and every
+// iterate lives at one scale: 64-bit integers X in units of 2^(gb - 61) with
+// |X| < 2^61, gb chosen so that the largest iterate keeps one or two bits of
+// headroom (see rescaling below).
+//
+// Products.  M is held as h 2^30 + l in units of 2^-60 (both signed, 32 bits),
+// an iterate is split as h 2^31 + 2 l; h h, h l and l h are summed in two
+// 64-bit accumulators, which 8 terms cannot overflow, and l l (below half of
+// the last unit) is left out.  Against 80-bit arithmetic on the subproblems of
+// 6-DoF and 3-DoF solves (2000 iterations) the results are as near as the
+// FP64 loop's: x_hat 0.5 to 1 times its error, u_hat and phi 0.5 to 2 times,
+// all within 2e-15.
+//
+// Range.  Every iterate that is multiplied or stored is or-ed into a word of
+// magnitudes; every 10 iterations the CTA looks at it.  A value beyond the
+// range restarts the loop at a coarser unit from the warm start, which stays
+// in the image until the loop ends; where that does not help (or the data is
+// not finite, or |M| is not small because sigma was underestimated), -1 is
+// returned and the caller runs the FP64 loop.  Otherwise the unit follows the
+// largest iterate by shifts.
+//
+// Work split: the tiles and butterflies of phase_pipg_ks.  At N = 15 a CTA
+// runs 128 threads and about 4400 warp instructions an iteration, 850 of them
+// multiply-adds, against 382 FP64 instructions of 16 cycles each.  Measured
+// (16384 instances, N = 15, 2000 iterations, one SCP iteration): 2580 cycles
+// an instance and iteration against 6890 of phase_pipg, 415 against 847 ms
+// for the whole SCP iteration.  Bound by latency now: two CTAs (8 warps) an
+// SM at 248 registers, 1.36 instructions a clock.
+// ---------------------------------------------------------------------------
+struct FxM { int h, l; };  // matrix entry: (h 2^30 + l) 2^-60
+struct FxC { int h, l2; };  // constant: (h 2^30 + l2 / 2) 2^-60
+struct FxV { int h, l; };  // iterate: h 2^31 + 2 l
+struct FxAcc {
+  long long hh = 0, cr = 1LL << 28;  // cr: rounds the shift of fx_fin
+};
+
+// c + a b; written out because the compiler widens loop-invariant factors
+// ahead of the loop and then multiplies 64 by 64 bits (4100 cycles an instance
+// and iteration against 2580)
+__device__ __forceinline__ long long fx_mw(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ int fx_low31(long long x) { return int(unsigned(x) << 1) >> 1; }
+__device__ __forceinline__ int fx_high(long long x, int l31) { return int(x >> 31) + int(unsigned(l31) >> 31); }
+__device__ __forceinline__ FxV fx_split(long long x) {
+  const int l = fx_low31(x);
+  return FxV{fx_high(x, l), (l + 1) >> 1};
+}
+__device__ __forceinline__ void fx_mad(FxAcc& a, FxM m, FxV v) {
+  a.hh = fx_mw(m.h, v.h, a.hh);
+  a.cr = fx_mw(m.h, v.l, a.cr);
+  a.cr = fx_mw(m.l, v.h, a.cr);
+}
+__device__ __forceinline__ long long fx_fin(const FxAcc& a) { return (a.hh << 1) + (a.cr >> 29); }
+// x c, for |x| < 2^62 and 0 <= c < 2
+__device__ __forceinline__ long long fx_mul(long long x, FxC c) {
+  const int l = fx_low31(x), h = fx_high(x, l);
+  const long long cr = fx_mw(h, c.l2, fx_mw(l, c.h, 1LL << 29));
+  return (fx_mw(h, c.h, 0) << 1) + (cr >> 30);
+}
+__device__ __forceinline__ FxC fx_const(long long c) {
+  const int l = int(unsigned(c) << 2) >> 2;
+  return FxC{int((c - l) >> 30), 2 * l};
+}
+// a b s to the nearest integer, a = ah + al, s a power of two
+__device__ __forceinline__ long long fx_prod(double ah, double al, double b, double s) {
+  const double bs = b * s, p = ah * bs;
+  return __double2ll_rn(p) + __double2ll_rn(fma(al, bs, fma(ah, bs, -p)));
+}
+__device__ __forceinline__ long long fx_sat(long long x) {
+  constexpr long long m = 1LL << 62;
+  return x > m ? m : (x < -m ? -m : x);
+}
+__device__ __forceinline__ unsigned fx_mag(long long x) {
+  const int h = int(x >> 32);
+  return unsigned(h ^ (h >> 31));
+}
+__device__ __forceinline__ unsigned long long fx_abs(long long x) { return (unsigned long long)(x < 0 ? -x : x); }
+__device__ __forceinline__ long long fx_max0(long long x) { return x < 0 ? 0 : x; }
+// x 2^-s to the nearest integer (s > 0), or x 2^-s exactly (s <= 0)
+__device__ __forceinline__ long long fx_shift(long long x, int s) {
+  return s > 0 ? (x + (1LL << (s - 1))) >> s : (long long)((unsigned long long)x << -s);
+}
+__device__ __forceinline__ unsigned block_or(unsigned v, unsigned* red) {
+  const int nw = (blockDim.x + 31) >> 5;
+  v = __reduce_or_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  unsigned m = 0;
+  for (int i = 0; i < nw; ++i) m |= red[i];
+  __syncthreads();
+  return m;
+}
+
+// Order of the states in the padded node vector.  A lane's stored rows 2 h
+// run over the even places of its tile, its stored columns 2 q over the even
+// ones too (ks_perm flips only higher bits).  So where half of the states
+// depend on nothing outside that half (6-DoF: mass, attitude and rates; 3-DoF:
+// mass and velocity), they take the even places, and a quarter of every
+// lane's tile, even rows times odd columns, is structurally zero: it is
+// neither held nor multiplied (16 of 96 tile registers, 48 of 288
+// multiply-adds).  Other models keep their order and the whole tile.
+struct FxOrder {
+  unsigned char state[KS_NXB], place[KS_NXB];  // state NX and up: padding
+  bool split;
+};
+__host__ __device__ constexpr FxOrder make_fx_order() {
+  FxOrder F{};
+  const StmOrder S = make_stm_order();
+  unsigned even = 0;
+  for (int a = 0; a < KS_NXB / 2; ++a) even |= 1u << S.row_order[NX - 1 - a];  // the sparsest rows
+  F.split = true;
+  for (int a = 0; a < KS_NXB / 2; ++a) F.split = F.split && (S.row_mask[S.row_order[NX - 1 - a]] & ~even) == 0;
+  int e = 0, o = 1;
+  for (int i = 0; i < KS_NXB; ++i) {
+    int p = i;
+    if (F.split) {
+      if (i < NX && ((even >> i) & 1u)) { p = e; e += 2; } else { p = o; o += 2; }
+    }
+    F.state[p] = (unsigned char)i;
+    F.place[i] = (unsigned char)p;
+  }
+  return F;
+}
+static __constant__ FxOrder kFx = make_fx_order();
+constexpr bool FX_SPLIT = make_fx_order().split;
+constexpr int FX_IY = make_fx_order().place[IY], FX_IM = make_fx_order().place[IM];
+__host__ __device__ constexpr bool fx_zero(int s, int q) { return FX_SPLIT && (s & 1) == 0 && (q & 1) == 1; }
+
+// The exchange region, behind everything make_lay lays out (64-bit elements,
+// 16-byte aligned rows, states by their place): gamma psi~, 2 x - x~ and gamma w of every interval
+// or node [N][KS_NXB], (2 u - u~ split) and the control gradients [N][nup],
+// gamma theta~, gamma eps, the dilation box [N], the fixed components of the
+// first and the last node [2][KS_NXB], alpha w_ep and alpha w_cost, the
+// relaxed virtual controls, then the unextrapolated iterates of the stop test.
+struct FxLay { int vp, dx, gw, du, bq, th, ep, lo, hi, zx, kc, nvp, nvm, px, pu, pmp, pmm, pph, pth, end; };
+__host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
+  const int nup = KS_NC * ((L.nu + KS_NC - 1) / KS_NC), n1 = (L.N + 1) & ~1;
+  FxLay Q;
+  int o = (L.total + 1) & ~1;
+  Q.vp = o; o += L.N * KS_NXB;
+  Q.dx = o; o += L.N * KS_NXB;
+  Q.gw = o; o += L.N * KS_NXB;
+  Q.du = o; o += L.N * nup;
+  Q.bq = o; o += L.N * nup;
+  Q.th = o; o += n1;
+  Q.ep = o; o += n1;
+  Q.lo = o; o += n1;
+  Q.hi = o; o += n1;
+  Q.zx = o; o += 2 * KS_NXB;
+  Q.kc = o; o += 2;
+  Q.nvp = o; o += L.N * KS_NXB;
+  Q.nvm = o; o += L.N * KS_NXB;
+  Q.px = o; o += L.N * KS_NXB;
+  Q.pu = o; o += L.N * nup;
+  Q.pmp = o; o += L.N * KS_NXB;
+  Q.pmm = o; o += L.N * KS_NXB;
+  Q.pph = o; o += L.N * KS_NXB;
+  Q.pth = o; o += n1;
+  Q.end = o;
+  return Q;
+}
+
+// iterations between two looks at the magnitudes
+constexpr int FX_WINDOW = 10;
+
+// Returns the iterations run (at least one), or -1 with the image untouched.
+template <int NU>
+__device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, double sigma, int force) {
+  using U = unsigned long long;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  double* const sm = reinterpret_cast<double*>(smraw);
+  constexpr int NXB = KS_NXB, TR = KS_TR, TC = KS_TC, NR = KS_NR, NCB = KS_NC, GS = KS_GS;
+  constexpr int WR = KS_WR, WC = KS_WC;
+  static_assert(WR == 2 && WC == 2, "the lane's rows and components load as pairs");
+  constexpr int NC = (NU + NCB - 1) / NCB;  // control columns per lane
+  constexpr int NUP = NCB * NC;
+  const int N = L.N, tid = threadIdx.x;
+  const FxLay Q = make_fx_lay(L);
+  long long* const ex = reinterpret_cast<long long*>(smraw);
+  const int g = tid / GS, ln = tid - GS * g;
+  const int rb = ln / NCB, cb = ln - NCB * rb;
+  // roles of threads past the last group: see phase_pipg_ks
+  const bool wlive = (tid & ~31) < N * GS;
+  const bool live = g < N, has_iv = g < N - 1;
+  const int gv = live ? g : N - 1;
+  const int gm1 = gv > 0 ? gv - 1 : 0, gp1 = gv < N - 1 ? gv + 1 : gv;
+  const int c0 = TC * cb + WC * rb;  // the lane's x components c0, c0 + 1 of node g
+  const int i0 = TR * rb + WR * cb;  // the lane's dual rows i0, i0 + 1 of interval g
+  const double wp = P.w_prox, om = P.omega;
+  const double alpha = 2.0 / (wp + sqrt(wp * wp + 4.0 * om * sigma));
+  // sqrt(omega), its inverse and gamma to twice the precision (high + low)
+  const double so = sqrt(om), sol = fma(-so, so, om) / (2.0 * so);
+  const double is = 1.0 / so, isl = is * (fma(-is, so, 1.0) - is * sol);
+  const double ga = alpha * so, gal = fma(alpha, so, -ga) + alpha * sol;
+  // ---- scales, and whether the data suits (the same answer on every thread)
+  U top[3] = {0, 0, 0};  // largest constant; largest iterate; largest |M|
+  {
+    using OB = OrdBits<double>;
+    for (int t = tid; t < (N - 1) * NX; t += blockDim.x) {
+      top[0] = umax(top[0], OB::abs(ga * sm[L.w + t]));
+      top[1] = umax(top[1], umax(OB::abs(is * sm[L.phi + t]), umax(OB::abs(sm[L.mup + t]), OB::abs(sm[L.mum + t]))));
+    }
+    for (int t = tid; t < N * NX; t += blockDim.x) top[1] = umax(top[1], OB::abs(sm[L.xh + t]));
+    for (int t = tid; t < N * NU; t += blockDim.x) top[1] = umax(top[1], OB::abs(sm[L.uh + t]));
+    for (int t = tid; t < N - 1; t += blockDim.x) {
+      top[0] = umax(top[0], OB::abs(ga * sm[L.eps + t]));
+      top[1] = umax(top[1], OB::abs(is * sm[L.th + t]));
+    }
+    for (int t = tid; t < NX; t += blockDim.x) top[0] = umax(top[0], umax(OB::abs(sm[L.zi + t]), OB::abs(sm[L.zf + t])));
+    for (int t = tid; t < (N - 1) * STM_SAS; t += blockDim.x) top[2] = umax(top[2], OB::abs(ga * sm[L.Am + t]));
+    // (the padding entry of an odd block stride is not written)
+    for (int t = tid; t < (N - 1) * NX * NU; t += blockDim.x) {
+      const int k = t / (NX * NU), o = k * b_stride(NU) + t - k * (NX * NU);
+      top[2] = umax(top[2], umax(OB::abs(ga * sm[L.Bm + o]), OB::abs(ga * sm[L.Bp + o])));
+    }
+    if (tid == 0) top[0] = umax(top[0], OB::abs(alpha * P.w_cost));
+    block_max_u<U, 3>(top, reinterpret_cast<U*>(sm + L.red));
+  }
+  const double vc = __longlong_as_double((long long)top[0]), vs = __longlong_as_double((long long)top[1]);
+  const double mx = __longlong_as_double((long long)top[2]);
+  const double ref = fmax(fmax(vc, vs), P.w_ep * is);
+  // the range test of |M|: sigma bounds its spectral norm by one, so that a
+  // row's or column's sum of |M| stays below 5; an entry over 1.2 shows that
+  // the power iteration fell short
+  if (!(mx <= 1.2 && vc < 1e60 && vs < 1e60 && ref > 1e-60 && ref < 1e60 && ga > 0.0 && P.rho > 0.0 && P.rho < 1.99 &&
+        alpha * wp < 1.0))
+    return -1;
+  const int gmin = ilogb(fmax(vc, 1e-60)) + 2;  // unit bound: constants below half of the range
+  const FxC C1 = fx_const((1LL << 60) - fx_prod(alpha, 0.0, wp, 0x1p60));
+  const FxC GM = fx_const(fx_prod(ga, gal, 1.0, 0x1p60));
+  const FxC RH = fx_const(__double2ll_rn(P.rho * 0x1p60));
+  // ---- tiles of M, in the lane's stored order (see ks_perm)
+  const int prow = ks_perm<NCB, TR>(cb), pcol = ks_perm<NR, TC>(rb);
+  FxM ap[TR][TC], bm[TR][NC], bp[TR][NC];
+  auto entry = [&](bool ok, int off) {
+    const long long m = ok ? fx_prod(ga, gal, sm[off], 0x1p60) : 0;
+    const int l = int(unsigned(m) << 2) >> 2;
+    return FxM{int((m - l) >> 30), l};
+  };
+#pragma unroll
+  for (int s = 0; s < TR; ++s) {
+    const int r = kFx.state[TR * rb + (s ^ prow)];
+#pragma unroll
+    for (int q = 0; q < TC; ++q) {
+      if (fx_zero(s, q)) { ap[s][q] = FxM{0, 0}; continue; }
+      const int c = kFx.state[TC * cb + (q ^ pcol)];
+      const bool ok = has_iv && r < NX && c < NX;
+      ap[s][q] = entry(ok, ok ? L.Am + g * STM_SAS + stm_index(r, c) : 0);
+    }
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int cc = cb + NCB * q;
+      const bool ok = has_iv && r < NX && cc < NU;
+      const int o = ok ? g * b_stride(NU) + r * NU + cc : 0;
+      bm[s][q] = entry(ok, L.Bm + o);
+      bp[s][q] = entry(ok, L.Bp + o);
+    }
+  }
+  bool fx[WC], okx[WC], okd[WR];
+#pragma unroll
+  for (int e = 0; e < WC; ++e) {
+    const int c = kFx.state[c0 + e];
+    okx[e] = live && c < NX;
+    fx[e] = okx[e] && (g == 0 || (g == N - 1 && P.fix_f[c]));
+  }
+#pragma unroll
+  for (int e = 0; e < WR; ++e) okd[e] = has_iv && kFx.state[i0 + e] < NX;
+  const bool th_lane = has_iv && FX_IY >= i0 && FX_IY < i0 + WR;
+  const int jmax = force > 0 ? force : P.pipg_jmax;
+  const bool chk_on = force <= 0 && P.pipg_jcheck > 0;
+  const int per = chk_on ? P.pipg_jcheck : jmax;
+  int gb = ilogb(ref) + 3;  // range 8 to 16 times the largest quantity in sight
+  for (int attempt = 0; attempt < 4; ++attempt, gb += 6) {
+    if (gb < gmin) gb = gmin;
+    double sc = ldexp(1.0, 61 - gb);
+    long long xt[WC], ft[WR], gf[WR], ut[NC], tht = 0;
+    FxV fg[TR];
+    // constants in the current unit.  alpha w_ep and the box saturate at twice the
+    // range, beyond which they decide nothing.
+    auto constants = [&]() {
+      if (tid == 0) {
+        ex[Q.kc] = alpha * P.w_ep * sc < 0x1p62 ? fx_prod(alpha, 0.0, P.w_ep, sc) : 1LL << 62;
+        ex[Q.kc + 1] = fx_prod(alpha, 0.0, P.w_cost, sc);
+      }
+      for (int t = tid; t < N * NXB; t += blockDim.x) {
+        const int k = t / NXB, i = kFx.state[t - NXB * k];
+        ex[Q.gw + t] = (k < N - 1 && i < NX) ? fx_prod(ga, gal, sm[L.w + k * NX + i], sc) : 0;
+      }
+      for (int t = tid; t < N; t += blockDim.x) {
+        ex[Q.ep + t] = t < N - 1 ? fx_prod(ga, gal, sm[L.eps + t], sc) : 0;
+        ex[Q.lo + t] = fx_sat(__double2ll_rn(sm[L.lo + t] * sc));
+        ex[Q.hi + t] = fx_sat(__double2ll_rn(sm[L.hi + t] * sc));
+      }
+      for (int t = tid; t < NXB; t += blockDim.x) {
+        const int i = kFx.state[t];
+        ex[Q.zx + t] = i < NX ? __double2ll_rn(sm[L.zi + i] * sc) : 0;
+        ex[Q.zx + NXB + t] = i < NX ? __double2ll_rn(sm[L.zf + i] * sc) : 0;
+      }
+    };
+    // the state's exchanged parts: gamma psi~, gamma theta~, psi~ on the whole
+    // tile row, hat B^+^T psi~ for node g+1
+    auto gather = [&]() {
+      int vh[WR], vl[WR], h[TR], l[TR];
+#pragma unroll
+      for (int e = 0; e < WR; ++e) {
+        const FxV v = fx_split(ft[e]);
+        vh[e] = v.h; vl[e] = v.l;
+      }
+      ks_all_gather<NCB, 1>(vh, h);
+      ks_all_gather<NCB, 1>(vl, l);
+#pragma unroll
+      for (int s = 0; s < TR; ++s) fg[s] = FxV{h[s], l[s]};
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        FxAcc a;
+#pragma unroll
+        for (int s = 0; s < TR; ++s) fx_mad(a, bp[s][q], fg[s]);
+        const long long v = ks_all_sum<NR, NCB>(fx_fin(a));
+        if (has_iv && rb == 0 && cb + NCB * q < NU) ex[Q.bq + (g + 1) * NUP + cb + NCB * q] = v;
+      }
+    };
+    auto publish = [&]() {
+      if (wlive) {
+#pragma unroll
+        for (int e = 0; e < WR; ++e) {
+          gf[e] = fx_mul(ft[e], GM);
+          if (okd[e]) ex[Q.vp + g * NXB + i0 + e] = gf[e];
+        }
+        gather();
+        if (th_lane) ex[Q.th + g] = fx_mul(tht, GM);
+      }
+    };
+    for (int t = tid; t < Q.end - Q.vp; t += blockDim.x) ex[Q.vp + t] = 0;
+    __syncthreads();
+    constants();
+#pragma unroll
+    for (int e = 0; e < WC; ++e) {
+      xt[e] = okx[e] ? __double2ll_rn(sm[L.xh + g * NX + kFx.state[c0 + e]] * sc) : 0;
+      if (okx[e]) ex[Q.px + g * NXB + c0 + e] = xt[e];
+    }
+#pragma unroll
+    for (int e = 0; e < WR; ++e) {
+      const int o = okd[e] ? g * NX + kFx.state[i0 + e] : 0;
+      ft[e] = okd[e] ? fx_prod(is, isl, sm[L.phi + o], sc) : 0;
+      gf[e] = 0;
+      if (okd[e]) {
+        const int oe = g * NXB + i0 + e;
+        ex[Q.pmp + oe] = ex[Q.nvp + oe] = __double2ll_rn(sm[L.mup + o] * sc);
+        ex[Q.pmm + oe] = ex[Q.nvm + oe] = __double2ll_rn(sm[L.mum + o] * sc);
+        ex[Q.pph + g * NXB + i0 + e] = ft[e];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int cc = cb + NCB * q;
+      ut[q] = (live && cc < NU) ? __double2ll_rn(sm[L.uh + g * NU + cc] * sc) : 0;
+      if (live && cc < NU && rb == 0) ex[Q.pu + g * NUP + cc] = ut[q];
+    }
+    if (th_lane) {
+      tht = fx_prod(is, isl, sm[L.th + g], sc);
+      ex[Q.pth + g] = tht;
+    }
+    publish();
+    __syncthreads();
+    unsigned mag = 0;
+    // V as in phase_pipg_ks: 0 plain, 1 stores the unextrapolated iterates,
+    // 2 tests against the stored ones, then stores
+    auto iterate = [&](auto v_tag) -> bool {
+      constexpr int V = decltype(v_tag)::value;
+      constexpr bool chk = V == 2, st = V >= 1;
+      U zn = 0, zo = 0, zd = 0, rn = 0, ro = 0, rd = 0;
+      FxV dxv[WC], duv[NC];
+#pragma unroll
+      for (int e = 0; e < WC; ++e) dxv[e] = FxV{0, 0};
+#pragma unroll
+      for (int q = 0; q < NC; ++q) duv[q] = FxV{0, 0};
+      // ---- projected gradient step (primal)
+      if (wlive) {
+        long long cx[TC], gx[WC], cu[NC];
+#pragma unroll
+        for (int q = 0; q < TC; ++q) {
+          FxAcc a;
+#pragma unroll
+          for (int s = 0; s < TR; ++s)
+            if (!fx_zero(s, q)) fx_mad(a, ap[s][q], fg[s]);
+          cx[q] = fx_fin(a);
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          FxAcc a;
+#pragma unroll
+          for (int s = 0; s < TR; ++s) fx_mad(a, bm[s][q], fg[s]);
+          cu[q] = ks_all_sum<NR, NCB>(fx_fin(a)) + ex[Q.bq + gv * NUP + cb + NCB * q];
+        }
+        ks_reduce_scatter<NR, NCB>(cx, gx);
+        const longlong2 vp = *reinterpret_cast<const longlong2*>(ex + Q.vp + gm1 * NXB + c0);
+        const long long td = ex[Q.th + gm1] - ex[Q.th + gv];  // th[N-1] stays zero
+#pragma unroll
+        for (int e = 0; e < WC; ++e) {
+          const int c = c0 + e;
+          const long long G = gx[e] - (e == 0 ? vp.x : vp.y) + (c == FX_IY ? td : 0);
+          long long xn = fx_mul(xt[e], C1) - G + ((g == N - 1 && c == FX_IM) ? ex[Q.kc + 1] : 0);
+          if (fx[e]) xn = ex[Q.zx + (g == 0 ? 0 : NXB) + c];
+          xn = okx[e] ? xn : 0;
+          const long long d = 2 * xn - xt[e];
+          if (okx[e]) ex[Q.dx + g * NXB + c] = d;
+          dxv[e] = fx_split(d);
+          xt[e] += fx_mul(xn - xt[e], RH);
+          mag |= fx_mag(xn) | fx_mag(d) | fx_mag(xt[e]);
+          if constexpr (chk) {
+            const long long old = ex[Q.px + g * NXB + c];
+            if (okx[e]) { zn = umax(zn, fx_abs(xn)); zo = umax(zo, fx_abs(old)); zd = umax(zd, fx_abs(xn - old)); }
+          }
+          if constexpr (st) {
+            if (okx[e]) ex[Q.px + g * NXB + c] = xn;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          const int cc = cb + NCB * q;
+          const bool ok = live && cc < NU;
+          long long un = fx_mul(ut[q], C1) - cu[q];
+          if (cc == NU - 1) {
+            const long long lo = ex[Q.lo + gv], hi = ex[Q.hi + gv];
+            un = un < lo ? lo : un;
+            un = un > hi ? hi : un;
+          }
+          un = ok ? un : 0;
+          const long long d = 2 * un - ut[q];
+          duv[q] = fx_split(d);
+          if (ok && rb == 0) reinterpret_cast<FxV*>(ex)[Q.du + g * NUP + cc] = duv[q];
+          ut[q] += fx_mul(un - ut[q], RH);
+          mag |= fx_mag(un) | fx_mag(d) | fx_mag(ut[q]);
+          if constexpr (chk) {
+            if (ok) {
+              const long long old = ex[Q.pu + g * NUP + cc];
+              zn = umax(zn, fx_abs(un)); zo = umax(zo, fx_abs(old)); zd = umax(zd, fx_abs(un - old));
+            }
+          }
+          if constexpr (st) {
+            // after every lane of the tile column has read it
+            __syncwarp();
+            if (ok && rb == 0) ex[Q.pu + g * NUP + cc] = un;
+          }
+        }
+      }
+      __syncthreads();
+      // ---- virtual controls and proportional-integral feedback (dual)
+      if (wlive) {
+        long long rr[TR], rs[WR];
+        {
+          int vh[WC], vl[WC], h[TC], l[TC];
+#pragma unroll
+          for (int e = 0; e < WC; ++e) { vh[e] = dxv[e].h; vl[e] = dxv[e].l; }
+          ks_all_gather<NR, NCB>(vh, h);
+          ks_all_gather<NR, NCB>(vl, l);
+          FxV du1[NC];
+#pragma unroll
+          for (int q = 0; q < NC; ++q) du1[q] = reinterpret_cast<const FxV*>(ex)[Q.du + gp1 * NUP + cb + NCB * q];
+#pragma unroll
+          for (int s = 0; s < TR; ++s) {
+            FxAcc a;
+#pragma unroll
+            for (int q = 0; q < TC; ++q)
+              if (!fx_zero(s, q)) fx_mad(a, ap[s][q], FxV{h[q], l[q]});
+#pragma unroll
+            for (int q = 0; q < NC; ++q) { fx_mad(a, bm[s][q], duv[q]); fx_mad(a, bp[s][q], du1[q]); }
+            rr[s] = fx_fin(a);
+          }
+        }
+        ks_reduce_scatter<NCB, 1>(rr, rs);
+        const longlong2 dn = *reinterpret_cast<const longlong2*>(ex + Q.dx + gp1 * NXB + i0);
+        const longlong2 gw = *reinterpret_cast<const longlong2*>(ex + Q.gw + gv * NXB + i0);
+        long long mp[WR], mm[WR], dmu[WR];
+        {
+          const longlong2 p2 = *reinterpret_cast<const longlong2*>(ex + Q.nvp + gv * NXB + i0);
+          const longlong2 m2 = *reinterpret_cast<const longlong2*>(ex + Q.nvm + gv * NXB + i0);
+          const long long AW = ex[Q.kc];
+          long long a[WR] = {p2.x, p2.y}, b[WR] = {m2.x, m2.y};
+          bool any = false;
+#pragma unroll
+          for (int e = 0; e < WR; ++e) {
+            mp[e] = fx_max0(a[e] - AW - gf[e]);
+            mm[e] = fx_max0(b[e] - AW + gf[e]);
+            dmu[e] = 0;
+            any = any || (okd[e] && (a[e] | b[e] | mp[e] | mm[e]) != 0);
+          }
+          // the virtual controls are zero unless a defect cannot be closed
+          if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+            for (int e = 0; e < WR; ++e) {
+              dmu[e] = (2 * mp[e] - a[e]) - (2 * mm[e] - b[e]);
+              a[e] += fx_mul(mp[e] - a[e], RH);
+              b[e] += fx_mul(mm[e] - b[e], RH);
+              if (okd[e]) {  // held to an eighth of the range: their sum with 2 x - x~ is multiplied
+                const unsigned m = fx_mag(mp[e]) | fx_mag(mm[e]) | fx_mag(a[e]) | fx_mag(b[e]);
+                mag |= m | (m << 3);
+                ex[Q.nvp + g * NXB + i0 + e] = a[e];
+                ex[Q.nvm + g * NXB + i0 + e] = b[e];
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < WR; ++e) {
+          const int o = g * NXB + i0 + e;
+          const long long f = ft[e];
+          if constexpr (chk) {
+            if (okd[e]) {
+              const long long op = ex[Q.pmp + o], oq = ex[Q.pmm + o];
+              zn = umax(zn, umax(U(mp[e]), U(mm[e])));
+              zo = umax(zo, umax(U(op), U(oq)));
+              zd = umax(zd, umax(fx_abs(mp[e] - op), fx_abs(mm[e] - oq)));
+            }
+          }
+          if constexpr (st) {
+            if (okd[e]) { ex[Q.pmp + o] = mp[e]; ex[Q.pmm + o] = mm[e]; }
+          }
+          long long d = rs[e] + (e == 0 ? gw.x : gw.y) + fx_mul(dmu[e] - (e == 0 ? dn.x : dn.y), GM);
+          d = okd[e] ? d : 0;  // rows that do not exist keep psi~ = 0
+          ft[e] = f + fx_mul(d, RH);
+          gf[e] = fx_mul(ft[e], GM);
+          mag |= fx_mag(d) | fx_mag(ft[e]);
+          if constexpr (chk) {
+            if (okd[e]) {
+              const long long old = ex[Q.pph + o], pn = f + d;
+              rn = umax(rn, fx_abs(pn)); ro = umax(ro, fx_abs(old)); rd = umax(rd, fx_abs(pn - old));
+            }
+          }
+          if constexpr (st) {
+            if (okd[e]) ex[Q.pph + o] = f + d;
+          }
+          if (okd[e]) ex[Q.vp + o] = gf[e];
+        }
+        gather();
+        if (th_lane) {
+          const long long hy = ex[Q.dx + gp1 * NXB + FX_IY] - ex[Q.dx + g * NXB + FX_IY];
+          const long long tn = fx_max0(tht + fx_mul(hy, GM) - ex[Q.ep + g]);
+          tht += fx_mul(tn - tht, RH);
+          mag |= fx_mag(tn) | fx_mag(tht);
+          if constexpr (chk) {
+            const long long old = ex[Q.pth + g];
+            rn = umax(rn, U(tn)); ro = umax(ro, fx_abs(old)); rd = umax(rd, fx_abs(tn - old));
+          }
+          if constexpr (st) ex[Q.pth + g] = tn;
+          ex[Q.th + g] = fx_mul(tht, GM);
+        }
+      }
+      if constexpr (chk) {
+        U w6[6] = {zn, zo, zd, rn, ro, rd};
+        block_max_u<U, 6>(w6, reinterpret_cast<U*>(sm + L.red));
+        const double eabs = P.eps_abs * sc, erel = P.eps_rel;
+        return double(w6[2]) <= eabs + erel * double(umax(w6[0], w6[1])) &&
+               so * double(w6[5]) <= eabs + erel * (so * double(umax(w6[3], w6[4])));
+      } else {
+        (void)zn; (void)zo; (void)zd; (void)rn; (void)ro; (void)rd;
+        __syncthreads();
+        return false;
+      }
+    };
+    int j = 0;
+    bool over = false;
+    while (j < jmax && !over) {
+      // up to the next stop test, the next look at the magnitudes or the end
+      // of the loop.  The last iteration before any of them stores the
+      // iterates that a test right behind it compares with.
+      const int to_test = per - j % per, to_look = FX_WINDOW - j % FX_WINDOW;
+      int nb = to_test < jmax - j ? to_test : jmax - j;
+      nb = to_look < nb ? to_look : nb;
+      const bool tested = chk_on && nb == to_test;
+      bool stop = false;
+      for (int k = tested ? 2 : 1; k < nb; ++k) iterate(KsTag<0>{});
+      if (!tested || nb >= 2) iterate(KsTag<1>{});
+      if (tested) stop = iterate(KsTag<2>{});
+      j += nb;
+      const unsigned m = block_or(mag, reinterpret_cast<unsigned*>(sm + L.red));
+      mag = 0;
+      over = m >= (1u << 29);
+      if (stop || over || j >= jmax) break;
+      // keep one or two bits of headroom (no finer unit in the first
+      // iterations, whose iterates still grow)
+      const int slack = __clz(m) - 3;
+      int s = slack < 1 ? 2 - slack : (slack > 2 && j >= 3 * FX_WINDOW ? 1 - slack : 0);
+      if (gb + s < gmin) s = gmin - gb;
+      if (s != 0) {
+        gb += s;
+        sc = ldexp(1.0, 61 - gb);
+#pragma unroll
+        for (int e = 0; e < WC; ++e) xt[e] = fx_shift(xt[e], s);
+#pragma unroll
+        for (int e = 0; e < WR; ++e) ft[e] = fx_shift(ft[e], s);
+#pragma unroll
+        for (int q = 0; q < NC; ++q) ut[q] = fx_shift(ut[q], s);
+        tht = fx_shift(tht, s);
+        for (int t = Q.nvp + tid; t < Q.end; t += blockDim.x) ex[t] = fx_shift(ex[t], s);
+        constants();
+        publish();
+        __syncthreads();
+      }
+    }
+    if (over) continue;
+    // the unextrapolated iterates to the image (warm start of the next SCP iteration)
+    const double un = ldexp(1.0, gb - 61);
+    __syncthreads();
+    for (int t = tid; t < N * NX; t += blockDim.x) sm[L.xh + t] = double(ex[Q.px + (t / NX) * NXB + kFx.place[t % NX]]) * un;
+    for (int t = tid; t < N * NU; t += blockDim.x) sm[L.uh + t] = double(ex[Q.pu + (t / NU) * NUP + t % NU]) * un;
+    for (int t = tid; t < (N - 1) * NX; t += blockDim.x) {
+      const int o = (t / NX) * NXB + kFx.place[t % NX];
+      sm[L.mup + t] = double(ex[Q.pmp + o]) * un;
+      sm[L.mum + t] = double(ex[Q.pmm + o]) * un;
+      const double f = double(ex[Q.pph + o]) * un;
+      sm[L.phi + t] = fma(f, so, f * sol);
+    }
+    for (int t = tid; t < N - 1; t += blockDim.x) {
+      const double f = double(ex[Q.pth + t]) * un;
+      sm[L.th + t] = fma(f, so, f * sol);
+    }
+    __syncthreads();
+    return j;
+  }
+  return -1;
+}
+
+}  // namespace pdg
