@@ -70,17 +70,23 @@ using namespace pdg;
 #ifndef PDG_KS_PERS_MAXT
 #define PDG_KS_PERS_MAXT 512
 #endif
-// The fixed-point loop of FP64 instances (internal variant 4): at most 256
-// threads (N = 32), so up to 255 registers for its tiles.
+// The fixed-point loop of FP64 instances runs 8 lanes a node (4 for NX <= 8):
+// internal variant 4 is built for up to 256 threads (N = 32), variant 5 for up
+// to 128 (N <= 16; 3-DoF N <= 32).  6-DoF takes two CTAs of 128 threads an SM
+// at 255 registers: three at 168 spill, are no faster on full batches (60.8
+// against 60.9 ms, 4096 instances, N = 15) and slower alone (7.6 against 7.1 ms,
+// 24 instances); four spill more (83 ms).  3-DoF's smaller tiles fit 168.
 #define PDG_FX_MAXT 256
+#define PDG_FX_MINB 1
+#define PDG_FX_MINB128 (pdg::NX <= 8 ? 3 : 2)
 #define PDG_LB_PERS(R, PV)                                                                  \
-  __launch_bounds__((PV) == 4 ? PDG_FX_MAXT : (PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT  \
+  __launch_bounds__((PV) >= 4 ? ((PV) == 4 ? PDG_FX_MAXT : 128) : (PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT  \
                     : ((PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512)), \
-                    sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
+                    (PV) >= 4 ? ((PV) == 4 ? PDG_FX_MINB : PDG_FX_MINB128) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 #define PDG_LB(R, PV)                                                                       \
-  __launch_bounds__((PV) == 4 ? PDG_FX_MAXT                                                   \
+  __launch_bounds__((PV) >= 4 ? ((PV) == 4 ? PDG_FX_MAXT : 128)                               \
                     : (PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512), \
-                    sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
+                    (PV) >= 4 ? ((PV) == 4 ? PDG_FX_MINB : PDG_FX_MINB128) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 
 namespace {
 
@@ -94,7 +100,7 @@ __device__ __noinline__ int pipg_fp64(const DParams& P, const Lay& L, double* sm
 template <typename R, int NU, int PV, bool CK = false>
 __device__ __forceinline__ int run_pipg(const DParams& P, const Lay& L, R* sm, R sigma, int force,
                                         double* ck = nullptr) {
-  if constexpr (PV == 4) {
+  if constexpr (PV >= 4) {
     const int it = phase_pipg_fx<NU>(P, L, sigma, force);
     return it >= 0 ? it : pipg_fp64<NU>(P, L, sm, sigma, force);
   } else if constexpr (PV == 2) return phase_pipg_reg<R, NU>(P, L, sm, sigma, force);
@@ -974,17 +980,20 @@ static int threads_for(int N, int nu, int precision) {
 // is an error.
 // The non-PIPG kernels of the plain form run with at most 512 threads.
 struct Plan {
-  int T;   // threads of the solve kernel (and of k_plain_pipg)
+  int T;   // threads of the solve kernel
   int Tr;  // threads of the other plain-form kernels
   int pv;  // 1 shared-memory PIPG, 2 register PIPG, 3 register tiles
-  int kv;  // the kernels' PIPG loop: pv, or 4 where form 1 runs in fixed point
+  // the plain form's PIPG kernel: its threads, and its PIPG loop as the solve
+  // kernel's (kv): pv, or 4, 5 where form 1 runs in fixed point
+  int Tp, kp;
+  int kv;
 };
 
 // Shared memory of a solve kernel for instances of up to N nodes with T threads.
 template <typename R>
 static size_t solve_smem(int N, int nu, int T, int kv) {
   const Lay L = make_lay(N, nu, T);
-  return (size_t)(kv == 4 ? make_fx_lay(L).end : L.total) * sizeof(R);
+  return (size_t)(kv >= 4 ? make_fx_lay(L).end : L.total) * sizeof(R);
 }
 
 static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bool use_override = true) {
@@ -1001,7 +1010,7 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
              " threads per CTA at N = " + std::to_string(N);
       return false;
     }
-    *out = {T, T < 512 ? T : 512, 2, 2};
+    *out = {T, T < 512 ? T : 512, 2, T, 2, 2};
   } else if (pv == 3) {
     // the lane groups' threads, at least two warps (the discretization wants
     // one interval per wave); the plain form's other kernels at least 128
@@ -1012,7 +1021,7 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
              " threads per CTA at N = " + std::to_string(N);
       return false;
     }
-    *out = {T, T < 128 ? 128 : T, 3, 3};
+    *out = {T, T < 128 ? 128 : T, 3, T, 3, 3};
   } else {
     // FP64 runs the loop in 64-bit fixed point (phase_pipg_fx: 5 to 8 times
     // the FP64 loop's rate at every N) wherever its lane groups and its
@@ -1024,7 +1033,10 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
     if (fx && ov == 0) T = T < tks ? tks : (T > PDG_FX_MAXT ? PDG_FX_MAXT : T);
     fx = fx && T >= tks && T <= PDG_FX_MAXT && solve_smem<double>(N, h->p.nu, T, 4) <= 226 * 1024;
     if (!fx && ov == 0) T = threads_for(N, h->p.nu, h->p.precision);
-    *out = {T, T, 1, fx ? 4 : 1};
+    // the plain form's PIPG kernel runs no more threads than its lane groups
+    // (3-DoF: 64 of the discretization's 128 at N = 15, so twice the CTAs)
+    const int Tp = !fx ? T : (tks < 64 ? 64 : tks);
+    *out = {T, T, 1, Tp, !fx ? 1 : Tp <= 128 ? 5 : 4, !fx ? 1 : T <= 128 ? 5 : 4};
   }
   return true;
 }
@@ -1040,14 +1052,14 @@ static PersistentFn<R, NU> persistent_fn(int pv, bool ck = false) {
     if (ck && pv == 1) return k_persistent<R, NU, 1, true>;
   }
   if constexpr (sizeof(R) == 8) {
-    if (pv == 4) return k_persistent<R, NU, 4>;
+    if (pv >= 4) return pv == 5 ? k_persistent<R, NU, 5> : k_persistent<R, NU, 4>;
   }
   return pv == 3 ? k_persistent<R, NU, 3> : (pv == 2 ? k_persistent<R, NU, 2> : k_persistent<R, NU, 1>);
 }
 template <typename R, int NU>
 static PlainPipgFn<R, NU> plain_pipg_fn(int pv) {
   if constexpr (sizeof(R) == 8) {
-    if (pv == 4) return k_plain_pipg<R, NU, 4>;
+    if (pv >= 4) return pv == 5 ? k_plain_pipg<R, NU, 5> : k_plain_pipg<R, NU, 4>;
   }
   return pv == 3 ? k_plain_pipg<R, NU, 3> : (pv == 2 ? k_plain_pipg<R, NU, 2> : k_plain_pipg<R, NU, 1>);
 }
@@ -1064,7 +1076,8 @@ struct Kern {
     for (const void* f : fns) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if constexpr (sizeof(R) == 8) {
       const void* fp64[] = {(const void*)k_persistent<R, NU, 1, true>, (const void*)k_persistent<R, NU, 4>,
-                            (const void*)k_plain_pipg<R, NU, 4>};
+                            (const void*)k_persistent<R, NU, 5>, (const void*)k_plain_pipg<R, NU, 4>,
+                            (const void*)k_plain_pipg<R, NU, 5>};
       for (const void* f : fp64) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     return 0;
@@ -1080,8 +1093,8 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   const int T = pl.T;
   const Lay L = make_lay(h->n_max, NU, T);
   // of the persistent kernel or the plain form's PIPG kernel, and of the plain form's others
-  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
-  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, pl.Tr) * sizeof(R);
+  const size_t smem = mode == 0 ? solve_smem<R>(h->n_max, NU, pl.Tp, pl.kp) : solve_smem<R>(h->n_max, NU, T, pl.kv);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, pl.Tp, pl.Tr) * sizeof(R);
   if (L.ipw < 1 || make_lay(h->n_max, NU, pl.Tr).ipw < 1)
     return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
   if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
@@ -1195,14 +1208,14 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   W.lit = h->lit;
   PDG_CUDA(h, cudaMemsetAsync(W.done, 0, sizeof(int), s));
   const int Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   k_plain_init<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
   PDG_CUDA(h, cudaGetLastError());
   cudaGraph_t graph = nullptr;
   PDG_CUDA(h, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
   k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
-  kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
+  kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
   k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters, pipg_iters,
                                              trace, nullptr);
   cudaError_t ce = cudaStreamEndCapture(s, &graph);
@@ -1271,11 +1284,11 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   std::string why;
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   h->last_variant = pl.pv;
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
-  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
+  const size_t smem = solve_smem<R>(h->n_max, NU, pl.Tp, pl.kp);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, pl.Tp, Tr) * sizeof(R);
   if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
   const size_t istride = (size_t)L.img;
   const size_t need = istride * sizeof(R) * B;
@@ -1313,7 +1326,7 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   k_pack<R, NU><<<B, 128, 0, s>>>(B, h->n_max, T, x0, Ns, W, 0, X, U, xh, uh, mup, mum, phi, th, sigma, defect, iters);
   k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
   k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, force);
-  kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, force);
+  kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, force);
   k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 1, nullptr, nullptr, nullptr, nullptr, nullptr,
                                              nullptr, nullptr, nullptr, step);
   k_pack<R, NU><<<B, 128, 0, s>>>(B, h->n_max, T, x0, Ns, W, 1, X, U, xh, uh, mup, mum, phi, th, sigma, defect, iters);
@@ -1349,10 +1362,10 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   std::string why;
   if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
-  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kv);
+  const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   const Lay L = make_lay(h->n_max, NU, T);
-  const size_t smem = solve_smem<R>(h->n_max, NU, T, pl.kv);
-  const size_t smem_r = (size_t)plain_total(h->n_max, NU, T, Tr) * sizeof(R);
+  const size_t smem = solve_smem<R>(h->n_max, NU, pl.Tp, pl.kp);
+  const size_t smem_r = (size_t)plain_total(h->n_max, NU, pl.Tp, Tr) * sizeof(R);
   if (L.ipw < 1) return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t istride = (size_t)L.img;
@@ -1388,7 +1401,7 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   for (int j = 0; j < h->p.scp_jmax; ++j) {
     k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
     k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
-    kpp<<<B, T, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
+    kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
     k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters,
                                                pipg_iters, nullptr, nullptr);
   }

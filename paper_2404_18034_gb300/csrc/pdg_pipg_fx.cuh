@@ -13,8 +13,8 @@ namespace pdg {
 // Variables.  With psi = phi / sqrt(omega), theta likewise, gamma = alpha
 // sqrt(omega) and M = gamma K, the iteration of Alg. PIPG_custom reads
 //   x' = c1 x~ - M^T psi~ + ...,  psi' = psi~ + M (2 x' - x~) + gamma (w + ...)
-// so one matrix M of spectral norm at most one serves both steps, and every
-// iterate lives at one scale: 64-bit integers X in units of 2^(gb - 61) with
+// so one matrix M of spectral norm at most one serves both steps (x and u are
+// held negated: the primal step then only adds), and every iterate lives at one scale: 64-bit integers X in units of 2^(gb - 61) with
 // |X| < 2^61, gb chosen so that the largest iterate keeps one or two bits of
 // headroom (see rescaling below).
 //
@@ -35,15 +35,17 @@ namespace pdg {
 // largest iterate by shifts.
 //
 // Work split: the tiles and butterflies of phase_pipg_ks.  At N = 15 a CTA
-// runs 128 threads and about 4400 warp instructions an iteration, 850 of them
+// runs 128 threads and about 4200 warp instructions an iteration, 900 of them
 // multiply-adds, against 382 FP64 instructions of 16 cycles each.  Measured
-// (16384 instances, N = 15, 2000 iterations, one SCP iteration): 2580 cycles
-// an instance and iteration against 6890 of phase_pipg, 415 against 847 ms
-// for the whole SCP iteration.  Bound by latency now: two CTAs (8 warps) an
-// SM at 248 registers, 1.36 instructions a clock.
+// (4096 instances, N = 15): 30.1 ms per 1000 iterations, 2330 cycles an
+// instance and iteration against 6890 of phase_pipg; N = 30 (1024 instances)
+// 15.9 ms.  Bound by latency and issue: two CTAs (8 warps) an SM at 255
+// registers, 1.5 instructions a clock; a third CTA at 168 registers adds
+// spills and no speed.
 // ---------------------------------------------------------------------------
 struct FxM { int h, l; };  // matrix entry: (h 2^30 + l) 2^-60
 struct FxC { int h, l2; };  // constant: (h 2^30 + l2 / 2) 2^-60
+struct FxR { int h, l; };   // relaxation less one: (h 2^31 + l) 2^-62
 struct FxV { int h, l; };  // iterate: h 2^31 + 2 l
 struct FxAcc {
   long long hh = 0, cr = 1LL << 28;  // cr: rounds the shift of fx_fin
@@ -51,7 +53,7 @@ struct FxAcc {
 
 // c + a b; written out because the compiler widens loop-invariant factors
 // ahead of the loop and then multiplies 64 by 64 bits (4100 cycles an instance
-// and iteration against 2580)
+// and iteration against 2580 in the first version of this loop)
 __device__ __forceinline__ long long fx_mw(int a, int b, long long c) {
   long long r;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
@@ -78,6 +80,15 @@ __device__ __forceinline__ long long fx_mul(long long x, FxC c) {
 __device__ __forceinline__ FxC fx_const(long long c) {
   const int l = int(unsigned(c) << 2) >> 2;
   return FxC{int((c - l) >> 30), 2 * l};
+}
+__device__ __forceinline__ FxM fx_entry(long long m) {
+  const int l = int(unsigned(m) << 2) >> 2;
+  return FxM{int((m - l) >> 30), l};
+}
+// x + (rho - 1) e: the relaxed iterate from the new one and its step
+__device__ __forceinline__ long long fx_relax(long long x, long long e, FxR r) {
+  const int l = fx_low31(e), h = fx_high(e, l);
+  return fx_mw(h, r.h, x) + (fx_mw(h, r.l, fx_mw(l, r.h, 1LL << 30)) >> 31);
 }
 // a b s to the nearest integer, a = ah + al, s a power of two
 __device__ __forceinline__ long long fx_prod(double ah, double al, double b, double s) {
@@ -145,10 +156,10 @@ constexpr int FX_IY = make_fx_order().place[IY], FX_IM = make_fx_order().place[I
 __host__ __device__ constexpr bool fx_zero(int s, int q) { return FX_SPLIT && (s & 1) == 0 && (q & 1) == 1; }
 
 // The exchange region, behind everything make_lay lays out (64-bit elements,
-// 16-byte aligned rows, states by their place): gamma psi~, 2 x - x~ and gamma w of every interval
-// or node [N][KS_NXB], (2 u - u~ split) and the control gradients [N][nup],
-// gamma theta~, gamma eps, the dilation box [N], the fixed components of the
-// first and the last node [2][KS_NXB], alpha w_ep and alpha w_cost, the
+// 16-byte aligned rows, states by their place): psi~ and 2 x - x~ (split) and gamma w of every interval
+// or node [N][KS_NXB], 2 u - u~ (split) and the control gradients [N][nup],
+// gamma theta~, gamma eps [N], the dilation box and, behind it, no box [N + 1], the fixed components of the
+// first and the last node [2][KS_NXB], alpha w_ep, alpha w_cost and zero, the
 // relaxed virtual controls, then the unextrapolated iterates of the stop test.
 struct FxLay { int vp, dx, gw, du, bq, th, ep, lo, hi, zx, kc, nvp, nvm, px, pu, pmp, pmm, pph, pth, end; };
 __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
@@ -162,10 +173,10 @@ __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
   Q.bq = o; o += L.N * nup;
   Q.th = o; o += n1;
   Q.ep = o; o += n1;
-  Q.lo = o; o += n1;
-  Q.hi = o; o += n1;
+  Q.lo = o; o += n1 + 2;
+  Q.hi = o; o += n1 + 2;
   Q.zx = o; o += 2 * KS_NXB;
-  Q.kc = o; o += 2;
+  Q.kc = o; o += 4;
   Q.nvp = o; o += L.N * KS_NXB;
   Q.nvm = o; o += L.N * KS_NXB;
   Q.px = o; o += L.N * KS_NXB;
@@ -244,16 +255,18 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         alpha * wp < 1.0))
     return -1;
   const int gmin = ilogb(fmax(vc, 1e-60)) + 2;  // unit bound: constants below half of the range
-  const FxC C1 = fx_const((1LL << 60) - fx_prod(alpha, 0.0, wp, 0x1p60));
   const FxC GM = fx_const(fx_prod(ga, gal, 1.0, 0x1p60));
-  const FxC RH = fx_const(__double2ll_rn(P.rho * 0x1p60));
+  FxR RL;
+  {
+    const long long c = __double2ll_rn((P.rho - 1.0) * 0x1p62);
+    RL.l = fx_low31(c);
+    RL.h = int((c - RL.l) >> 31);
+  }
   // ---- tiles of M, in the lane's stored order (see ks_perm)
   const int prow = ks_perm<NCB, TR>(cb), pcol = ks_perm<NR, TC>(rb);
   FxM ap[TR][TC], bm[TR][NC], bp[TR][NC];
   auto entry = [&](bool ok, int off) {
-    const long long m = ok ? fx_prod(ga, gal, sm[off], 0x1p60) : 0;
-    const int l = int(unsigned(m) << 2) >> 2;
-    return FxM{int((m - l) >> 30), l};
+    return fx_entry(ok ? fx_prod(ga, gal, sm[off], 0x1p60) : 0);
   };
 #pragma unroll
   for (int s = 0; s < TR; ++s) {
@@ -274,16 +287,28 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
       bp[s][q] = entry(ok, L.Bp + o);
     }
   }
-  bool fx[WC], okx[WC], okd[WR];
+  // scalar entries, zero on the lanes of groups that hold no such quantity:
+  // 1 - alpha w_prox for x~ and (on the first tile row) u~, gamma for the -I
+  // blocks next to hat A^-
+  const long long c1 = (1LL << 60) - fx_prod(alpha, 0.0, wp, 0x1p60), g1 = fx_prod(ga, gal, 1.0, 0x1p60);
+  const FxM cx1 = fx_entry(live ? c1 : 0), cu1 = fx_entry(live && rb == 0 ? c1 : 0);
+  const FxM gxm = fx_entry(live ? -g1 : 0), gdm = fx_entry(has_iv ? -g1 : 0);
+  bool fx[WC];
 #pragma unroll
   for (int e = 0; e < WC; ++e) {
     const int c = kFx.state[c0 + e];
-    okx[e] = live && c < NX;
-    fx[e] = okx[e] && (g == 0 || (g == N - 1 && P.fix_f[c]));
+    fx[e] = live && c < NX && (g == 0 || (g == N - 1 && P.fix_f[c]));
   }
-#pragma unroll
-  for (int e = 0; e < WR; ++e) okd[e] = has_iv && kFx.state[i0 + e] < NX;
+  const bool okx[WC] = {live && kFx.state[c0] < NX, live && kFx.state[c0 + 1] < NX};
+  const bool okd[WR] = {has_iv && kFx.state[i0] < NX, has_iv && kFx.state[i0 + 1] < NX};
   const bool th_lane = has_iv && FX_IY >= i0 && FX_IY < i0 + WR;
+  // where the lane finds what most lanes do not have (then a zero): the CTCS
+  // duals of its y component, the cost of its mass, its dilation box
+  const bool y_lane = live && FX_IY >= c0 && FX_IY < c0 + WC;
+  const int tha = y_lane ? gm1 : N - 1, thb = y_lane ? gv : N - 1;
+  const int kcm = (g == N - 1 && FX_IM >= c0 && FX_IM < c0 + WC) ? 1 : 2;
+  const int box = cb + NCB * (NC - 1) == NU - 1 ? gv : N;
+  const int gq = live ? g : 0;  // (node 1 has no control gradient from before it)
   const int jmax = force > 0 ? force : P.pipg_jmax;
   const bool chk_on = force <= 0 && P.pipg_jcheck > 0;
   const int per = chk_on ? P.pipg_jcheck : jmax;
@@ -291,14 +316,21 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
   for (int attempt = 0; attempt < 4; ++attempt, gb += 6) {
     if (gb < gmin) gb = gmin;
     double sc = ldexp(1.0, 61 - gb);
-    long long xt[WC], ft[WR], gf[WR], ut[NC], tht = 0;
+    long long xt[WC], ft[WR], ut[NC], tht = 0;
     FxV fg[TR];
+    unsigned psi_t = 0;  // |psi| below this (in units of 2^32) leaves virtual controls of zero at zero
     // constants in the current unit.  alpha w_ep and the box saturate at twice the
     // range, beyond which they decide nothing.
     auto constants = [&]() {
+      const double pt = P.w_ep * is * sc;
+      psi_t = pt < 0x1p62 ? unsigned((long long)pt >> 32) : 0x7fffffffu;
+      psi_t = psi_t > 0 ? psi_t - 1 : 0;
       if (tid == 0) {
         ex[Q.kc] = alpha * P.w_ep * sc < 0x1p62 ? fx_prod(alpha, 0.0, P.w_ep, sc) : 1LL << 62;
-        ex[Q.kc + 1] = fx_prod(alpha, 0.0, P.w_cost, sc);
+        ex[Q.kc + 1] = -fx_prod(alpha, 0.0, P.w_cost, sc);
+        ex[Q.kc + 2] = 0;
+        ex[Q.lo + N] = -(1LL << 62);
+        ex[Q.hi + N] = 1LL << 62;
       }
       for (int t = tid; t < N * NXB; t += blockDim.x) {
         const int k = t / NXB, i = kFx.state[t - NXB * k];
@@ -306,17 +338,17 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
       }
       for (int t = tid; t < N; t += blockDim.x) {
         ex[Q.ep + t] = t < N - 1 ? fx_prod(ga, gal, sm[L.eps + t], sc) : 0;
-        ex[Q.lo + t] = fx_sat(__double2ll_rn(sm[L.lo + t] * sc));
-        ex[Q.hi + t] = fx_sat(__double2ll_rn(sm[L.hi + t] * sc));
+        ex[Q.lo + t] = -fx_sat(__double2ll_rn(sm[L.hi + t] * sc));
+        ex[Q.hi + t] = -fx_sat(__double2ll_rn(sm[L.lo + t] * sc));
       }
       for (int t = tid; t < NXB; t += blockDim.x) {
         const int i = kFx.state[t];
-        ex[Q.zx + t] = i < NX ? __double2ll_rn(sm[L.zi + i] * sc) : 0;
-        ex[Q.zx + NXB + t] = i < NX ? __double2ll_rn(sm[L.zf + i] * sc) : 0;
+        ex[Q.zx + t] = i < NX ? -__double2ll_rn(sm[L.zi + i] * sc) : 0;
+        ex[Q.zx + NXB + t] = i < NX ? -__double2ll_rn(sm[L.zf + i] * sc) : 0;
       }
     };
-    // the state's exchanged parts: gamma psi~, gamma theta~, psi~ on the whole
-    // tile row, hat B^+^T psi~ for node g+1
+    // the state's exchanged parts: psi~ for node g+1 and on the whole tile row,
+    // hat B^+^T psi~ for node g+1
     auto gather = [&]() {
       int vh[WR], vl[WR], h[TR], l[TR];
 #pragma unroll
@@ -324,6 +356,7 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         const FxV v = fx_split(ft[e]);
         vh[e] = v.h; vl[e] = v.l;
       }
+      if (live) *reinterpret_cast<int4*>(ex + Q.vp + g * NXB + i0) = make_int4(vh[0], vl[0], vh[1], vl[1]);
       ks_all_gather<NCB, 1>(vh, h);
       ks_all_gather<NCB, 1>(vl, l);
 #pragma unroll
@@ -339,11 +372,6 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
     };
     auto publish = [&]() {
       if (wlive) {
-#pragma unroll
-        for (int e = 0; e < WR; ++e) {
-          gf[e] = fx_mul(ft[e], GM);
-          if (okd[e]) ex[Q.vp + g * NXB + i0 + e] = gf[e];
-        }
         gather();
         if (th_lane) ex[Q.th + g] = fx_mul(tht, GM);
       }
@@ -353,14 +381,13 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
     constants();
 #pragma unroll
     for (int e = 0; e < WC; ++e) {
-      xt[e] = okx[e] ? __double2ll_rn(sm[L.xh + g * NX + kFx.state[c0 + e]] * sc) : 0;
+      xt[e] = okx[e] ? -__double2ll_rn(sm[L.xh + g * NX + kFx.state[c0 + e]] * sc) : 0;
       if (okx[e]) ex[Q.px + g * NXB + c0 + e] = xt[e];
     }
 #pragma unroll
     for (int e = 0; e < WR; ++e) {
       const int o = okd[e] ? g * NX + kFx.state[i0 + e] : 0;
       ft[e] = okd[e] ? fx_prod(is, isl, sm[L.phi + o], sc) : 0;
-      gf[e] = 0;
       if (okd[e]) {
         const int oe = g * NXB + i0 + e;
         ex[Q.pmp + oe] = ex[Q.nvp + oe] = __double2ll_rn(sm[L.mup + o] * sc);
@@ -371,7 +398,7 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       const int cc = cb + NCB * q;
-      ut[q] = (live && cc < NU) ? __double2ll_rn(sm[L.uh + g * NU + cc] * sc) : 0;
+      ut[q] = (live && cc < NU) ? -__double2ll_rn(sm[L.uh + g * NU + cc] * sc) : 0;
       if (live && cc < NU && rb == 0) ex[Q.pu + g * NUP + cc] = ut[q];
     }
     if (th_lane) {
@@ -381,6 +408,17 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
     publish();
     __syncthreads();
     unsigned mag = 0;
+    // the largest |psi~| of the lane's rows, and whether the warp holds a
+    // virtual control that is not zero
+    unsigned pm = umax(fx_mag(ft[0]), fx_mag(ft[1]));
+    bool nz = false;
+    if (wlive) {
+      bool any = false;
+#pragma unroll
+      for (int e = 0; e < WR; ++e)
+        any = any || (okd[e] && (ex[Q.nvp + g * NXB + i0 + e] | ex[Q.nvm + g * NXB + i0 + e]) != 0);
+      nz = __any_sync(0xffffffffu, any);
+    }
     // V as in phase_pipg_ks: 0 plain, 1 stores the unextrapolated iterates,
     // 2 tests against the stored ones, then stores
     auto iterate = [&](auto v_tag) -> bool {
@@ -395,12 +433,17 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
       // ---- projected gradient step (primal)
       if (wlive) {
         long long cx[TC], gx[WC], cu[NC];
+        const int4 vp = *reinterpret_cast<const int4*>(ex + Q.vp + gm1 * NXB + c0);
 #pragma unroll
         for (int q = 0; q < TC; ++q) {
           FxAcc a;
 #pragma unroll
           for (int s = 0; s < TR; ++s)
             if (!fx_zero(s, q)) fx_mad(a, ap[s][q], fg[s]);
+          if (q < WC) {  // the sums that stay on this lane also take x~ and the -I block
+            fx_mad(a, cx1, fx_split(xt[q]));
+            fx_mad(a, gxm, q == 0 ? FxV{vp.x, vp.y} : FxV{vp.z, vp.w});
+          }
           cx[q] = fx_fin(a);
         }
 #pragma unroll
@@ -408,46 +451,47 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
           FxAcc a;
 #pragma unroll
           for (int s = 0; s < TR; ++s) fx_mad(a, bm[s][q], fg[s]);
-          cu[q] = ks_all_sum<NR, NCB>(fx_fin(a)) + ex[Q.bq + gv * NUP + cb + NCB * q];
+          fx_mad(a, cu1, fx_split(ut[q]));
+          cu[q] = ks_all_sum<NR, NCB>(fx_fin(a)) + ex[Q.bq + gq * NUP + cb + NCB * q];
         }
         ks_reduce_scatter<NR, NCB>(cx, gx);
-        const longlong2 vp = *reinterpret_cast<const longlong2*>(ex + Q.vp + gm1 * NXB + c0);
-        const long long td = ex[Q.th + gm1] - ex[Q.th + gv];  // th[N-1] stays zero
+        gx[FX_IY & 1] += ex[Q.th + tha] - ex[Q.th + thb];  // th[N-1] stays zero
+        gx[FX_IM & 1] += ex[Q.kc + kcm];
+        int dv[2 * WC];
 #pragma unroll
         for (int e = 0; e < WC; ++e) {
           const int c = c0 + e;
-          const long long G = gx[e] - (e == 0 ? vp.x : vp.y) + (c == FX_IY ? td : 0);
-          long long xn = fx_mul(xt[e], C1) - G + ((g == N - 1 && c == FX_IM) ? ex[Q.kc + 1] : 0);
+          long long xn = gx[e];
           if (fx[e]) xn = ex[Q.zx + (g == 0 ? 0 : NXB) + c];
-          xn = okx[e] ? xn : 0;
-          const long long d = 2 * xn - xt[e];
-          if (okx[e]) ex[Q.dx + g * NXB + c] = d;
+          const long long st_ = xn - xt[e], d = xn + st_;
           dxv[e] = fx_split(d);
-          xt[e] += fx_mul(xn - xt[e], RH);
+          dv[2 * e] = dxv[e].h;
+          dv[2 * e + 1] = dxv[e].l;
+          xt[e] = fx_relax(xn, st_, RL);
           mag |= fx_mag(xn) | fx_mag(d) | fx_mag(xt[e]);
           if constexpr (chk) {
-            const long long old = ex[Q.px + g * NXB + c];
+            const long long old = okx[e] ? ex[Q.px + g * NXB + c] : 0;
             if (okx[e]) { zn = umax(zn, fx_abs(xn)); zo = umax(zo, fx_abs(old)); zd = umax(zd, fx_abs(xn - old)); }
           }
           if constexpr (st) {
             if (okx[e]) ex[Q.px + g * NXB + c] = xn;
           }
         }
+        if (live) *reinterpret_cast<int4*>(ex + Q.dx + g * NXB + c0) = make_int4(dv[0], dv[1], dv[2], dv[3]);
 #pragma unroll
         for (int q = 0; q < NC; ++q) {
           const int cc = cb + NCB * q;
           const bool ok = live && cc < NU;
-          long long un = fx_mul(ut[q], C1) - cu[q];
-          if (cc == NU - 1) {
-            const long long lo = ex[Q.lo + gv], hi = ex[Q.hi + gv];
+          long long un = cu[q];
+          if (q == NC - 1) {
+            const long long lo = ex[Q.lo + box], hi = ex[Q.hi + box];
             un = un < lo ? lo : un;
             un = un > hi ? hi : un;
           }
-          un = ok ? un : 0;
-          const long long d = 2 * un - ut[q];
+          const long long st_ = un - ut[q], d = un + st_;
           duv[q] = fx_split(d);
           if (ok && rb == 0) reinterpret_cast<FxV*>(ex)[Q.du + g * NUP + cc] = duv[q];
-          ut[q] += fx_mul(un - ut[q], RH);
+          ut[q] = fx_relax(un, st_, RL);
           mag |= fx_mag(un) | fx_mag(d) | fx_mag(ut[q]);
           if constexpr (chk) {
             if (ok) {
@@ -466,6 +510,8 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
       // ---- virtual controls and proportional-integral feedback (dual)
       if (wlive) {
         long long rr[TR], rs[WR];
+        const int4 dn = *reinterpret_cast<const int4*>(ex + Q.dx + gp1 * NXB + i0);
+        const longlong2 gw = *reinterpret_cast<const longlong2*>(ex + Q.gw + gv * NXB + i0);
         {
           int vh[WC], vl[WC], h[TC], l[TC];
 #pragma unroll
@@ -483,46 +529,42 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
               if (!fx_zero(s, q)) fx_mad(a, ap[s][q], FxV{h[q], l[q]});
 #pragma unroll
             for (int q = 0; q < NC; ++q) { fx_mad(a, bm[s][q], duv[q]); fx_mad(a, bp[s][q], du1[q]); }
+            if (s < WR) fx_mad(a, gdm, s == 0 ? FxV{dn.x, dn.y} : FxV{dn.z, dn.w});
             rr[s] = fx_fin(a);
           }
         }
         ks_reduce_scatter<NCB, 1>(rr, rs);
-        const longlong2 dn = *reinterpret_cast<const longlong2*>(ex + Q.dx + gp1 * NXB + i0);
-        const longlong2 gw = *reinterpret_cast<const longlong2*>(ex + Q.gw + gv * NXB + i0);
-        long long mp[WR], mm[WR], dmu[WR];
-        {
-          const longlong2 p2 = *reinterpret_cast<const longlong2*>(ex + Q.nvp + gv * NXB + i0);
-          const longlong2 m2 = *reinterpret_cast<const longlong2*>(ex + Q.nvm + gv * NXB + i0);
+        long long d[WR] = {gw.x - rs[0], gw.y - rs[1]};
+        long long mp[WR] = {0, 0}, mm[WR] = {0, 0};
+        // the virtual controls are zero unless a defect cannot be closed
+        if (nz || __any_sync(0xffffffffu, pm >= psi_t)) {
           const long long AW = ex[Q.kc];
-          long long a[WR] = {p2.x, p2.y}, b[WR] = {m2.x, m2.y};
           bool any = false;
 #pragma unroll
           for (int e = 0; e < WR; ++e) {
-            mp[e] = fx_max0(a[e] - AW - gf[e]);
-            mm[e] = fx_max0(b[e] - AW + gf[e]);
-            dmu[e] = 0;
-            any = any || (okd[e] && (a[e] | b[e] | mp[e] | mm[e]) != 0);
-          }
-          // the virtual controls are zero unless a defect cannot be closed
-          if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-            for (int e = 0; e < WR; ++e) {
-              dmu[e] = (2 * mp[e] - a[e]) - (2 * mm[e] - b[e]);
-              a[e] += fx_mul(mp[e] - a[e], RH);
-              b[e] += fx_mul(mm[e] - b[e], RH);
-              if (okd[e]) {  // held to an eighth of the range: their sum with 2 x - x~ is multiplied
-                const unsigned m = fx_mag(mp[e]) | fx_mag(mm[e]) | fx_mag(a[e]) | fx_mag(b[e]);
-                mag |= m | (m << 3);
-                ex[Q.nvp + g * NXB + i0 + e] = a[e];
-                ex[Q.nvm + g * NXB + i0 + e] = b[e];
-              }
+            if (okd[e]) {
+              const int o = g * NXB + i0 + e;
+              long long a = ex[Q.nvp + o], b = ex[Q.nvm + o];
+              const long long gf = fx_mul(ft[e], GM);
+              mp[e] = fx_max0(a - AW - gf);
+              mm[e] = fx_max0(b - AW + gf);
+              d[e] += fx_mul((2 * mp[e] - a) - (2 * mm[e] - b), GM);
+              a = fx_relax(mp[e], mp[e] - a, RL);
+              b = fx_relax(mm[e], mm[e] - b, RL);
+              ex[Q.nvp + o] = a;
+              ex[Q.nvm + o] = b;
+              any = any || (a | b) != 0;
+              // held to an eighth of the range: their sum is multiplied
+              const unsigned m = fx_mag(mp[e]) | fx_mag(mm[e]) | fx_mag(a) | fx_mag(b);
+              mag |= m | (m << 3);
             }
           }
+          nz = __any_sync(0xffffffffu, any);
         }
+        pm = 0;
 #pragma unroll
         for (int e = 0; e < WR; ++e) {
           const int o = g * NXB + i0 + e;
-          const long long f = ft[e];
           if constexpr (chk) {
             if (okd[e]) {
               const long long op = ex[Q.pmp + o], oq = ex[Q.pmm + o];
@@ -534,27 +576,30 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
           if constexpr (st) {
             if (okd[e]) { ex[Q.pmp + o] = mp[e]; ex[Q.pmm + o] = mm[e]; }
           }
-          long long d = rs[e] + (e == 0 ? gw.x : gw.y) + fx_mul(dmu[e] - (e == 0 ? dn.x : dn.y), GM);
-          d = okd[e] ? d : 0;  // rows that do not exist keep psi~ = 0
-          ft[e] = f + fx_mul(d, RH);
-          gf[e] = fx_mul(ft[e], GM);
-          mag |= fx_mag(d) | fx_mag(ft[e]);
+          const long long pn = ft[e] + d[e];
+          ft[e] = fx_relax(pn, d[e], RL);
+          const unsigned m = fx_mag(ft[e]);
+          pm = umax(pm, m);
+          mag |= fx_mag(d[e]) | m;
           if constexpr (chk) {
             if (okd[e]) {
-              const long long old = ex[Q.pph + o], pn = f + d;
+              const long long old = ex[Q.pph + o];
               rn = umax(rn, fx_abs(pn)); ro = umax(ro, fx_abs(old)); rd = umax(rd, fx_abs(pn - old));
             }
           }
           if constexpr (st) {
-            if (okd[e]) ex[Q.pph + o] = f + d;
+            if (okd[e]) ex[Q.pph + o] = pn;
           }
-          if (okd[e]) ex[Q.vp + o] = gf[e];
         }
         gather();
         if (th_lane) {
-          const long long hy = ex[Q.dx + gp1 * NXB + FX_IY] - ex[Q.dx + g * NXB + FX_IY];
-          const long long tn = fx_max0(tht + fx_mul(hy, GM) - ex[Q.ep + g]);
-          tht += fx_mul(tn - tht, RH);
+          const FxV ya = reinterpret_cast<const FxV*>(ex)[Q.dx + g * NXB + FX_IY];
+          const FxV yb = reinterpret_cast<const FxV*>(ex)[Q.dx + gp1 * NXB + FX_IY];
+          FxAcc a;
+          fx_mad(a, gdm, yb);
+          fx_mad(a, FxM{-gdm.h, -gdm.l}, ya);
+          const long long tn = fx_max0(tht + fx_fin(a) - ex[Q.ep + g]);
+          tht = fx_relax(tn, tn - tht, RL);
           mag |= fx_mag(tn) | fx_mag(tht);
           if constexpr (chk) {
             const long long old = ex[Q.pth + g];
@@ -610,6 +655,7 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
 #pragma unroll
         for (int q = 0; q < NC; ++q) ut[q] = fx_shift(ut[q], s);
         tht = fx_shift(tht, s);
+        pm = umax(fx_mag(ft[0]), fx_mag(ft[1]));
         for (int t = Q.nvp + tid; t < Q.end; t += blockDim.x) ex[t] = fx_shift(ex[t], s);
         constants();
         publish();
@@ -620,8 +666,8 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
     // the unextrapolated iterates to the image (warm start of the next SCP iteration)
     const double un = ldexp(1.0, gb - 61);
     __syncthreads();
-    for (int t = tid; t < N * NX; t += blockDim.x) sm[L.xh + t] = double(ex[Q.px + (t / NX) * NXB + kFx.place[t % NX]]) * un;
-    for (int t = tid; t < N * NU; t += blockDim.x) sm[L.uh + t] = double(ex[Q.pu + (t / NU) * NUP + t % NU]) * un;
+    for (int t = tid; t < N * NX; t += blockDim.x) sm[L.xh + t] = -double(ex[Q.px + (t / NX) * NXB + kFx.place[t % NX]]) * un;
+    for (int t = tid; t < N * NU; t += blockDim.x) sm[L.uh + t] = -double(ex[Q.pu + (t / NU) * NUP + t % NU]) * un;
     for (int t = tid; t < (N - 1) * NX; t += blockDim.x) {
       const int o = (t / NX) * NXB + kFx.place[t % NX];
       sm[L.mup + t] = double(ex[Q.pmp + o]) * un;

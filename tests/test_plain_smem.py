@@ -25,4 +25,4 @@ def test_plain_launches_hold_every_layout(tmp_path, defs):
     assert r.returncode == 0 and r.stdout.startswith("OK"), r.stdout
     assert int(r.stdout.split()[2]) > 0  # grids where PIPG's own layout is too small
     host = open(os.path.join(SRC, "pdg_mc.cu")).read()
-    assert host.count("plain_total(h->n_max, NU, T, ") == 3  # solve, step and no-allocation entry points
+    assert host.count("plain_total(h->n_max, NU, pl.Tp, ") == 3  # solve, step and no-allocation entry points
