@@ -58,6 +58,9 @@ struct Lay {
   int xt, ut, nup, num, vph, vth, dx, du, td, stage, red, total;
 };
 
+// a compile-time index as a function argument
+template <int V> struct IntTag { static constexpr int value = V; };
+
 }  // namespace pdg
 
 // The model -- F, g, their compact Jacobians and the initial guess of one
@@ -85,6 +88,9 @@ struct Lay {
 //               (the closure of df/dx's pattern under the flow).  The PIPG
 //               products then skip the entries outside the mask; without it
 //               every entry counts.
+// Optionally (PDG_MODEL_HAS_COLUMN_CLASSES defined, needs the STM mask), the
+// STM's columns by their rows, which the discretization by column classes
+// integrates without the zeros; see pdg_model_6dof.cuh for the interface.
 #if defined(PDG_MODEL_HEADER)
 #include PDG_MODEL_HEADER
 #elif defined(PDG_MODEL_3DOF)

@@ -378,6 +378,33 @@ k_plain_disc(const DParams P, int B, int Nmax, const int* __restrict__ Ns, Plain
   if (threadIdx.x == 0) img[L.sc + 1] = defect;
 }
 
+#ifdef PDG_MODEL_HAS_COLUMN_CLASSES
+// The same by column classes (discretize_cols), for models that declare them;
+// built for up to MAXT threads.  Two CTAs an SM: one is slower (18.6 against
+// 17.5 ms for an SCP iteration with 20 PIPG iterations, 4096 instances, N = 15;
+// FP32, 16384 instances: 9.3 against 6.3), three are no faster.
+template <typename R, int NU, int MAXT>
+__global__ void __launch_bounds__(MAXT, 2)
+k_plain_disc_cols(const DParams P, int B, int Nmax, const int* __restrict__ Ns, PlainWs W) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  R* sm = reinterpret_cast<R*>(smraw);
+  const int b = blockIdx.x;
+  if (W.st[b] != ST_RUNNING) return;
+  if (plain_aborted(P)) return;  // k_plain_update ends the instance
+  const int N = Ns ? Ns[b] : Nmax;
+  const Lay L = make_lay(N, NU, 128);
+  DiscColsLay D = make_disc_cols_lay(L, Nmax);
+  R* img = reinterpret_cast<R*>(W.img) + (size_t)b * W.istride;
+  copy_g2s(sm + L.x0, img + L.x0, L.Am - L.x0);  // x0, Xb, Ub
+  __syncthreads();
+  const R defect = discretize_cols<R, NU>(P, L, sm, D);
+  phase_scale_extra<R, NU>(P, L, sm);
+  __syncthreads();
+  copy_s2g(img + L.Am, sm + L.Am, L.xh - L.Am);  // Am .. zf
+  if (threadIdx.x == 0) img[L.sc + 1] = defect;
+}
+#endif
+
 template <typename R, int NU>
 __global__ void __launch_bounds__(512, sizeof(R) == 4 ? PDG_FP32_MIN_BLOCKS : 1)
 k_plain_power(const DParams P, int B, int Nmax, const int* __restrict__ Ns, PlainWs W, const int* force) {
@@ -1074,6 +1101,11 @@ struct Kern {
                          (const void*)k_plain_pipg<R, NU, 3>, (const void*)k_plain_update<R, NU>,
                          (const void*)k_subproblem<R, NU>};
     for (const void* f : fns) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+#ifdef PDG_MODEL_HAS_COLUMN_CLASSES
+    const size_t smem_d = make_disc_cols_lay(make_lay(h->n_max, NU, 128), h->n_max).total * sizeof(R);
+    const void* disc[] = {(const void*)k_plain_disc_cols<R, NU, 384>, (const void*)k_plain_disc_cols<R, NU, 512>};
+    for (const void* f : disc) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d));
+#endif
     if constexpr (sizeof(R) == 8) {
       const void* fp64[] = {(const void*)k_persistent<R, NU, 1, true>, (const void*)k_persistent<R, NU, 4>,
                             (const void*)k_persistent<R, NU, 5>, (const void*)k_plain_pipg<R, NU, 4>,
@@ -1083,6 +1115,23 @@ struct Kern {
     return 0;
   }
 };
+
+// The plain form's discretization: by column classes where the model declares them.
+template <typename R, int NU>
+static void launch_plain_disc(const DParams& dp, int B, int n_max, const int* Ns, const PlainWs& W, int Tr,
+                              size_t smem_r, cudaStream_t s) {
+#ifdef PDG_MODEL_HAS_COLUMN_CLASSES
+  (void)Tr;
+  (void)smem_r;
+  const DiscColsLay D = make_disc_cols_lay(make_lay(n_max, NU, 128), n_max);
+  const int T = 32 * disc_cols_warps(D.cap, NU);
+  const size_t smem = (size_t)D.total * sizeof(R);
+  if (T <= 384) k_plain_disc_cols<R, NU, 384><<<B, T, smem, s>>>(dp, B, n_max, Ns, W);
+  else k_plain_disc_cols<R, NU, 512><<<B, T, smem, s>>>(dp, B, n_max, Ns, W);
+#else
+  k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(dp, B, n_max, Ns, W);
+#endif
+}
 
 template <typename R, int NU>
 static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int mode, double* X, double* U, double* tf,
@@ -1213,7 +1262,7 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   PDG_CUDA(h, cudaGetLastError());
   cudaGraph_t graph = nullptr;
   PDG_CUDA(h, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-  k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+  launch_plain_disc<R, NU>(h->dp, B, h->n_max, Ns, W, Tr, smem_r, s);
   k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
   kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
   k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters, pipg_iters,
@@ -1324,7 +1373,7 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
   W.done = h->ints + 4 * (size_t)B;
   W.lit = h->lit;
   k_pack<R, NU><<<B, 128, 0, s>>>(B, h->n_max, T, x0, Ns, W, 0, X, U, xh, uh, mup, mum, phi, th, sigma, defect, iters);
-  k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+  launch_plain_disc<R, NU>(h->dp, B, h->n_max, Ns, W, Tr, smem_r, s);
   k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, force);
   kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, force);
   k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 1, nullptr, nullptr, nullptr, nullptr, nullptr,
@@ -1399,7 +1448,7 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
   PDG_CUDA(h, cudaMemsetAsync(W.done, 0, sizeof(int), s));
   k_plain_init<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, x0, Ns, W, X, U, tf, fuel, status, scp_iters, pipg_iters);
   for (int j = 0; j < h->p.scp_jmax; ++j) {
-    k_plain_disc<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W);
+    launch_plain_disc<R, NU>(h->dp, B, h->n_max, Ns, W, Tr, smem_r, s);
     k_plain_power<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
     kpp<<<B, pl.Tp, smem, s>>>(h->dp, B, h->n_max, Ns, W, nullptr);
     k_plain_update<R, NU><<<B, Tr, smem_r, s>>>(h->dp, B, h->n_max, Ns, W, 0, X, U, tf, fuel, status, scp_iters,

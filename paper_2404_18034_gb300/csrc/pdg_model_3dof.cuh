@@ -113,6 +113,40 @@ __device__ __forceinline__ void model_jvp(const R* __restrict__ A, const R* __re
   }
 }
 
+// The STM's columns by what they can hold, as in the 6-DoF model: m, r and v
+// one by one, y stays the unit vector.
+#define PDG_MODEL_HAS_COLUMN_CLASSES 1
+constexpr int COL_CLASSES = 0;
+__host__ __device__ constexpr int col_class_first(int) { return 0; }
+__host__ __device__ constexpr int col_class_size(int) { return 0; }
+constexpr int COL_SINGLES = 7;  // columns 0 .. 6
+constexpr int SA_Y = 4;  // first slot of the compact y row
+
+template <typename R, unsigned ROWS, unsigned ACT, typename Up>
+__device__ __forceinline__ void model_col_rows(const R* __restrict__ A, const R (&S)[NX], Up&& up) {
+  auto t = [&](auto j, R a, R acc) {
+    constexpr int J = decltype(j)::value;
+    if constexpr ((ROWS >> J) & 1u) return fma(a, S[J], acc);
+    else return acc;
+  };
+#define PDG_T(j, a, acc) t(IntTag<(j)>{}, (a), (acc))
+  {
+    R d = PDG_T(0, A[4], R(0));
+    d = PDG_T(1, A[5], d); d = PDG_T(2, A[9], d); d = PDG_T(3, A[10], d);
+    d = PDG_T(4, A[6], d); d = PDG_T(5, A[7], d); d = PDG_T(6, A[8], d);
+    up(7, d);
+  }
+  if constexpr ((ACT >> 1) & 1u) up(1, PDG_T(4, A[0], R(0)));
+  if constexpr ((ACT >> 2) & 1u) up(2, PDG_T(5, A[0], R(0)));
+  if constexpr ((ACT >> 3) & 1u) up(3, PDG_T(6, A[0], R(0)));
+  if constexpr ((ACT >> 4) & 7u) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) up(4 + i, PDG_T(0, A[1 + i], R(0)));
+  }
+  if constexpr (ACT & 1u) up(0, R(0));
+#undef PDG_T
+}
+
 // xb += (df/dx)^T v, ub += (df/du)^T v from a compact stage buffer (the
 // transpose of model_jvp).
 template <int NU>

@@ -199,6 +199,70 @@ __device__ __forceinline__ void model_jvp(const R* __restrict__ A, const R* __re
   }
 }
 
+// The STM's columns by what they can hold (see the discretization by column
+// classes): columns 7..10 (q) and 11..13 (w) as two classes whose columns
+// share one set of rows, columns m, r, v one by one, y not at all (it stays
+// the unit vector).
+#define PDG_MODEL_HAS_COLUMN_CLASSES 1
+constexpr int COL_CLASSES = 2;
+__host__ __device__ constexpr int col_class_first(int k) { return k == 0 ? IQ : IW; }
+__host__ __device__ constexpr int col_class_size(int k) { return k == 0 ? 4 : 3; }
+constexpr int COL_SINGLES = 7;  // columns 0 .. 6
+constexpr int SA_Y = 29;  // first slot of the compact y row
+
+// d = (df/dx) S for an S that is zero outside the rows of the mask ROWS, row by
+// row in an order that lets `up` overwrite S with the row's next stage: a row
+// is handed over when no later row reads it (y reads all, r reads v, v reads
+// m and q, q reads q and w, w reads w).  Only rows of the mask ACT are formed;
+// the others of ROWS do not change.
+template <typename R, unsigned ROWS, unsigned ACT, typename Up>
+__device__ __forceinline__ void model_col_rows(const R* __restrict__ A, const R (&S)[NX], Up&& up) {
+  auto t = [&](auto j, R a, R acc) {
+    constexpr int J = decltype(j)::value;
+    if constexpr ((ROWS >> J) & 1u) return fma(a, S[J], acc);
+    else return acc;
+  };
+#define PDG_T(j, a, acc) t(IntTag<(j)>{}, (a), (acc))
+  {
+    R d = PDG_T(0, A[29], R(0));
+    d = PDG_T(1, A[30], d); d = PDG_T(2, A[39], d); d = PDG_T(3, A[40], d);
+    d = PDG_T(4, A[31], d); d = PDG_T(5, A[32], d); d = PDG_T(6, A[33], d);
+    d = PDG_T(9, A[34], d); d = PDG_T(10, A[35], d);
+    d = PDG_T(11, A[36], d); d = PDG_T(12, A[37], d); d = PDG_T(13, A[38], d);
+    up(14, d);
+  }
+  if constexpr ((ACT >> 1) & 1u) up(1, PDG_T(4, A[0], R(0)));
+  if constexpr ((ACT >> 2) & 1u) up(2, PDG_T(5, A[0], R(0)));
+  if constexpr ((ACT >> 3) & 1u) up(3, PDG_T(6, A[0], R(0)));
+  if constexpr ((ACT >> 4) & 7u) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      R d = PDG_T(0, A[1 + i], R(0));
+      d = PDG_T(7, A[4 + 4 * i], d); d = PDG_T(8, A[5 + 4 * i], d);
+      d = PDG_T(9, A[6 + 4 * i], d); d = PDG_T(10, A[7 + 4 * i], d);
+      up(4 + i, d);
+    }
+  }
+  if constexpr ((ACT >> 7) & 0xFu) {
+    const R hw0 = A[16], hw1 = A[17], hw2 = A[18], hq0 = A[19], hq1 = A[20], hq2 = A[21], hq3 = A[22];
+    R e0 = PDG_T(8, -hw0, R(0)), e1 = PDG_T(7, hw0, R(0)), e2 = PDG_T(7, hw1, R(0)), e3 = PDG_T(7, hw2, R(0));
+    e0 = PDG_T(9, -hw1, e0); e1 = PDG_T(9, hw2, e1); e2 = PDG_T(8, -hw2, e2); e3 = PDG_T(8, hw1, e3);
+    e0 = PDG_T(10, -hw2, e0); e1 = PDG_T(10, -hw1, e1); e2 = PDG_T(10, hw0, e2); e3 = PDG_T(9, -hw0, e3);
+    e0 = PDG_T(11, -hq1, e0); e1 = PDG_T(11, hq0, e1); e2 = PDG_T(11, hq3, e2); e3 = PDG_T(11, -hq2, e3);
+    e0 = PDG_T(12, -hq2, e0); e1 = PDG_T(12, -hq3, e1); e2 = PDG_T(12, hq0, e2); e3 = PDG_T(12, hq1, e3);
+    e0 = PDG_T(13, -hq3, e0); e1 = PDG_T(13, hq2, e1); e2 = PDG_T(13, -hq1, e2); e3 = PDG_T(13, hq0, e3);
+    up(7, e0); up(8, e1); up(9, e2); up(10, e3);
+  }
+  if constexpr ((ACT >> 11) & 7u) {
+    const R e0 = PDG_T(13, A[24], PDG_T(12, A[23], R(0)));
+    const R e1 = PDG_T(13, A[26], PDG_T(11, A[25], R(0)));
+    const R e2 = PDG_T(12, A[28], PDG_T(11, A[27], R(0)));
+    up(11, e0); up(12, e1); up(13, e2);
+  }
+  if constexpr (ACT & 1u) up(0, R(0));
+#undef PDG_T
+}
+
 // xb += (df/dx)^T v, ub += (df/du)^T v from a compact stage buffer (the
 // transpose of model_jvp).
 template <int NU>

@@ -176,6 +176,337 @@ __device__ PDG_DISC_ATTR R phase_discretize(const DParams& P, const Lay& L, R* s
   return discretize_body<R, NU>(P, L, sm);
 }
 
+// ---------------------------------------------------------------------------
+// The discretization by column classes (its own kernel, k_plain_disc_cols).
+//
+// The FP64 pipe charges per warp instruction, whatever its active lanes, so
+// what counts is the instructions a warp issues for the columns it holds.
+// discretize_body gives every column the whole of df/dx times a column and
+// evaluates the model for as few intervals as its other warps hold columns
+// of (4 of 32 lanes at N = 15 in 128 threads).  Here
+//  * a CTA has a warp for every kind of column over all intervals of a wave
+//    (16 at nu = 4): the 2 NU control columns, the model's column classes
+//    (6-DoF: q and w), and one warp whose lanes hold all of an interval's
+//    remaining columns (m, r, v: few rows each) one after another; each runs
+//    the products its rows can hold and no others;
+//  * a stage forms df/dx S row by row in an order that lets a row's next
+//    stage overwrite S at once, so no separate derivative is kept;
+//  * the model is evaluated for all the wave's intervals at once, one stage
+//    ahead of the columns, in two warps: one the part of the Jacobians that
+//    does not depend on the path constraints, one the dynamics, the CTCS row
+//    and x.
+// In FP64 a stage lasts as long as the fullest of the SM's four schedulers
+// (warp % 4) needs for its share of the pipe: 64 cycles a warp instruction.
+// disc_role deals the warps out so that each gets about 300 of the 1215
+// instructions of a stage (6-DoF, nu = 4): F 290, Jacobians 200, a control warp
+// 100, w 81, q 54, single columns 55.  Two CTAs an SM fill each other's
+// barriers; the spills this costs (80 registers) stay off the FP64 pipe.
+// Measured (4096 instances, N = 15, 6-DoF, nu = 4, FP64): 12.1 ms against 25.6
+// of k_plain_disc, the FP64 pipe 87 % busy (one CTA an SM and the model in one
+// warp: 15.9 ms, 58 %); FP32, 16384 instances: 4.7 ms.
+// ---------------------------------------------------------------------------
+#ifdef PDG_MODEL_HAS_COLUMN_CLASSES
+// What warp i of a CTA does for a wave with U warps of control columns and C
+// warps of column classes: 'U' or 'C' (and which), 'F' dynamics and x, 'J' the
+// Jacobians, 'M' the single columns, '-' nothing.
+struct DiscRole { char kind; int index; };
+__host__ __device__ constexpr DiscRole disc_role(int warp, int U, int C) {
+  constexpr char order[13] = "UFCJUMCUU-CC";  // four of U and C each
+  if (warp >= 12) {
+    const int u = 4 + warp - 12, c = 4 + warp - 12 - (U > 4 ? U - 4 : 0);
+    return u < U ? DiscRole{'U', u} : (c < C ? DiscRole{'C', c} : DiscRole{'-', 0});
+  }
+  const char k = order[warp];
+  int n = 0;
+  for (int i = 0; i < warp; ++i) n += order[i] == k ? 1 : 0;
+  if ((k == 'U' && n >= U) || (k == 'C' && n >= C)) return DiscRole{'-', 0};
+  return DiscRole{k, n};
+}
+__host__ __device__ constexpr int disc_control_warps(int w, int nu) { return (2 * nu * w + 31) / 32; }
+__host__ __device__ constexpr int disc_class_warps(int w) {
+  int n = 0;
+  for (int k = 0; k < COL_CLASSES; ++k) n += (col_class_size(k) * w + 31) / 32;
+  return n;
+}
+// warps of the CTA for a wave of w intervals
+__host__ __device__ constexpr int disc_cols_warps(int w, int nu) {
+  const int U = disc_control_warps(w, nu), C = disc_class_warps(w);
+  int n = 12 + (U > 4 ? U - 4 : 0) + (C > 4 ? C - 4 : 0);
+  while (disc_role(n - 1, U, C).kind == '-') --n;
+  return n;
+}
+// intervals of a wave: up to 16, as many as 16 warps hold columns of
+__host__ __device__ constexpr int disc_cols_cap(int N, int nu) {
+  int w = N - 1 < 16 ? N - 1 : 16;
+  while (w > 1 && disc_cols_warps(w, nu) > 16) --w;
+  return w;
+}
+// Shared memory (elements): the image up to the subproblem's end, the stage
+// buffers at an odd stride (a warp's lanes read one entry of consecutive
+// intervals), the reduction's scratch.
+struct DiscColsLay { int cap, sa, stage, red, total; };
+__host__ __device__ inline DiscColsLay make_disc_cols_lay(const Lay& L, int n_max) {
+  DiscColsLay D;
+  D.cap = disc_cols_cap(n_max, L.nu);
+  D.sa = (2 * (SA_A + NX * L.nu) + 4 * NX) | 1;  // two Jacobian buffers; x: base, accumulator, two stage inputs
+  D.stage = L.xh;
+  D.red = D.stage + D.cap * D.sa;
+  D.total = D.red + 32;
+  return D;
+}
+
+__host__ __device__ constexpr unsigned col_rows(int c) {
+  unsigned m = 0;
+  for (int i = 0; i < NX; ++i) m |= stm_nz(i, c) ? 1u << i : 0u;
+  return m;
+}
+
+// RK4 state of one STM column: base, stage input, accumulator (entries outside
+// its rows are never used)
+template <typename R>
+struct ColState { R P[NX], S[NX], A[NX]; };
+
+// stage G of an RK4 step of the rows ACT; with INH, lam (df/du) e_cu is added
+template <typename R, int NU, int G, unsigned ROWS, unsigned ACT, bool INH>
+__device__ __forceinline__ void col_stage(ColState<R>& C, const R* J, R h, R h2, R h6, R lam, int cu) {
+  const R* Bd = J + SA_A + cu;
+  model_col_rows<R, ROWS, ACT>(J, C.S, [&](int i, R d) {
+    if constexpr (INH) d = fma(lam, Bd[i * NU], d);
+    if constexpr (G == 0) { C.A[i] = d; C.S[i] = fma(h2, d, C.P[i]); }
+    else if constexpr (G == 1) { C.A[i] = fma(R(2), d, C.A[i]); C.S[i] = fma(h2, d, C.P[i]); }
+    else if constexpr (G == 2) { C.A[i] = fma(R(2), d, C.A[i]); C.S[i] = fma(h, d, C.P[i]); }
+    else { C.P[i] = fma(h6, C.A[i] + d, C.P[i]); C.S[i] = C.P[i]; }
+  });
+}
+
+// One wave of a column warp: the unit vector of column c (or zero), every
+// stage with the evaluator's Jacobians, a barrier each.
+template <typename R, int NU, unsigned ROWS, unsigned ACT, bool INH>
+__device__ __forceinline__ void col_wave(ColState<R>& C, int c, const R* st, int nsub, R h, bool active, bool minus,
+                                         int cu) {
+  constexpr int JS = SA_A + NX * NU;
+  const R h2 = R(0.5) * h, h6 = h / R(6);
+#pragma unroll
+  for (int i = 0; i < NX; ++i) C.P[i] = C.S[i] = (i == c) ? R(1) : R(0);
+  __syncthreads();
+#pragma unroll 1
+  for (int n = 0; n < nsub; ++n) {
+    const R l0 = R(n) / R(nsub), l1 = (R(n) + R(0.5)) / R(nsub), l2 = R(n + 1) / R(nsub);
+    if (active) col_stage<R, NU, 0, ROWS, ACT, INH>(C, st, h, h2, h6, minus ? R(1) - l0 : l0, cu);
+    __syncthreads();
+    if (active) col_stage<R, NU, 1, ROWS, ACT, INH>(C, st + JS, h, h2, h6, minus ? R(1) - l1 : l1, cu);
+    __syncthreads();
+    if (active) col_stage<R, NU, 2, ROWS, ACT, INH>(C, st, h, h2, h6, minus ? R(1) - l1 : l1, cu);
+    __syncthreads();
+    if (active) col_stage<R, NU, 3, ROWS, ACT, INH>(C, st + JS, h, h2, h6, minus ? R(1) - l2 : l2, cu);
+    __syncthreads();
+  }
+}
+
+template <typename R, int NU>
+__device__ __forceinline__ void store_state_col(const DParams& P, const Lay& L, R* sm, int k, int c, unsigned rows,
+                                                const ColState<R>& C) {
+  const R pc = R(P.Px[c]);
+#pragma unroll
+  for (int i = 0; i < NX; ++i)
+    if ((rows >> i) & 1u) sm[L.Am + k * STM_SAS + stm_index(i, c)] = C.P[i] * pc * R(P.Pxinv[i]);
+}
+
+// the single columns C0 .. COL_SINGLES - 1 of one interval, one after another
+template <typename R, int NU, int G, int C0>
+__device__ __forceinline__ void singles_stage(ColState<R> (&C)[COL_SINGLES], const R* J, R h, R h2, R h6) {
+  if constexpr (C0 < COL_SINGLES) {
+    col_stage<R, NU, G, col_rows(C0), col_rows(C0) & ~(1u << C0), false>(C[C0], J, h, h2, h6, R(0), 0);
+    singles_stage<R, NU, G, C0 + 1>(C, J, h, h2, h6);
+  }
+}
+template <typename R, int NU, int C0>
+__device__ __forceinline__ void singles_store(const DParams& P, const Lay& L, R* sm, int k, const ColState<R> (&C)[COL_SINGLES]) {
+  if constexpr (C0 < COL_SINGLES) {
+    store_state_col<R, NU>(P, L, sm, k, C0, col_rows(C0), C[C0]);
+    singles_store<R, NU, C0 + 1>(P, L, sm, k, C);
+  }
+}
+
+// a column class's warp over the wave (its columns have the rows of the first)
+template <typename R, int NU, int K>
+__device__ __forceinline__ void class_wave(const DParams& P, const Lay& L, R* sm, const DiscColsLay& D, int task, int W,
+                                           int k0, R h) {
+  constexpr unsigned ROWS = col_rows(col_class_first(K));
+  const int ci = task / W, k = k0 + task - ci * W, c = col_class_first(K) + ci;
+  const bool active = ci < col_class_size(K) && k < L.N - 1;
+  ColState<R> C;
+  col_wave<R, NU, ROWS, ROWS, false>(C, c, sm + D.stage + (active ? k - k0 : 0) * D.sa, P.nsub, h, active, false, 0);
+  if (active) store_state_col<R, NU>(P, L, sm, k, c, ROWS, C);
+}
+// the class that worker wk (counted from the first class's) serves
+template <typename R, int NU, int K>
+__device__ __forceinline__ bool classes_wave(const DParams& P, const Lay& L, R* sm, const DiscColsLay& D, int wk, int W,
+                                             int k0, R h) {
+  if constexpr (K < COL_CLASSES) {
+    const int n = (col_class_size(K) * W + 31) / 32;
+    if (wk < n) {
+      class_wave<R, NU, K>(P, L, sm, D, wk * 32 + (threadIdx.x & 31), W, k0, h);
+      return true;
+    }
+    return classes_wave<R, NU, K + 1>(P, L, sm, D, wk - n, W, k0, h);
+  } else {
+    return false;
+  }
+}
+
+// Called by every thread of a CTA of disc_cols_warps(D.cap, NU) warps.
+template <typename R, int NU>
+__device__ __forceinline__ R discretize_cols(const DParams& P, const Lay& L, R* sm, const DiscColsLay& D) {
+  constexpr int JS = SA_A + NX * NU;
+  const int N = L.N, nsub = P.nsub;
+  const R* Xb = sm + L.Xb;
+  const R* Ub = sm + L.Ub;
+  const R h = R(1) / (R(N - 1) * R(nsub));
+  const R h2 = R(0.5) * h, h6 = h / R(6);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nw = (N - 1 + D.cap - 1) / D.cap, W = (N - 1 + nw - 1) / nw;  // waves of equal size
+  const DiscRole role = disc_role(warp, disc_control_warps(W, NU), disc_class_warps(W));
+  const int S = 4 * nsub;
+  // stage s of an interval: its time, its controls
+  auto stage_u = [&](int s, int k, R (&u)[NU]) {
+    const int g = s & 3;
+    const R lp = (R(s >> 2) + (g == 0 ? R(0) : (g == 3 ? R(1) : R(0.5)))) / R(nsub);
+#pragma unroll
+    for (int i = 0; i < NU; ++i) u[i] = (R(1) - lp) * Ub[k * NU + i] + lp * Ub[(k + 1) * NU + i];
+  };
+  R dmax = 0;
+  for (int k0 = 0; k0 < N - 1; k0 += W) {
+    if (role.kind == 'J') {  // df/dx and df/du but for the CTCS row and the dilation's column
+      const int k = k0 + lane;
+      const bool active = lane < W && k < N - 1;
+      R* st = sm + D.stage + (active ? lane : 0) * D.sa;
+      auto jac = [&](int s) {
+        R u[NU], x[NX], f[NX];
+        stage_u(s, k, u);
+        const R* xs = s == 0 ? Xb + k * NX : st + 2 * JS + (2 + (s & 1)) * NX;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) x[i] = xs[i];
+        R* J = st + (s & 1) * JS;
+        R A[SA_A], Bd[NX * NU];
+        model_eval<R, NU>(P, x, u, f, A, Bd);  // forms only what is stored
+#pragma unroll
+        for (int i = 0; i < SA_Y; ++i) J[i] = A[i];
+#pragma unroll
+        for (int i = 0; i < IY; ++i)
+#pragma unroll
+          for (int c = 0; c < NU - 1; ++c) J[SA_A + i * NU + c] = Bd[i * NU + c];
+      };
+      if (active) jac(0);
+      __syncthreads();
+#pragma unroll 1
+      for (int s = 0; s < S; ++s) {
+        if (active && s + 1 < S) jac(s + 1);
+        __syncthreads();
+      }
+    } else if (role.kind == 'F') {  // x, and of the Jacobians the CTCS row and the dilation's column
+      const int k = k0 + lane;
+      const bool active = lane < W && k < N - 1;
+      R* const st = sm + D.stage + (active ? lane : 0) * D.sa;
+      R* const xP = st + 2 * JS;
+      R* const xA = xP + NX;
+      // x's RK4 stage s: from its stage input to that of stage s + 1 (the
+      // Jacobians' warp reads the other one meanwhile)
+      auto x_stage = [&](int s) {
+        const int g = s & 3;
+        R u[NU], x[NX], d[NX], A[SA_A], Bd[NX * NU];
+        stage_u(s, k, u);
+        const R* xs = s == 0 ? xP : xA + (1 + (s & 1)) * NX;
+        R* xn = xA + (1 + ((s + 1) & 1)) * NX;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) x[i] = xs[i];
+        model_eval<R, NU>(P, x, u, d, A, Bd);  // forms only what is stored
+        R* J = st + (s & 1) * JS;
+#pragma unroll
+        for (int i = SA_Y; i < SA_A; ++i) J[i] = A[i];
+#pragma unroll
+        for (int i = 0; i < NX; ++i) J[SA_A + i * NU + NU - 1] = Bd[i * NU + NU - 1];
+#pragma unroll
+        for (int c = 0; c < NU - 1; ++c) J[SA_A + IY * NU + c] = Bd[IY * NU + c];
+        if (g == 3) {
+#pragma unroll
+          for (int i = 0; i < NX; ++i) { const R v = xP[i] + h6 * (xA[i] + d[i]); xP[i] = v; xn[i] = v; }
+        } else {
+          const R hs = g == 2 ? h : h2;
+#pragma unroll
+          for (int i = 0; i < NX; ++i) { xA[i] = g == 0 ? d[i] : fma(R(2), d[i], xA[i]); xn[i] = fma(hs, d[i], xP[i]); }
+        }
+      };
+      if (active) {
+#pragma unroll
+        for (int i = 0; i < NX; ++i) xP[i] = Xb[k * NX + i];
+        x_stage(0);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int s = 0; s < S; ++s) {
+        if (active && s + 1 < S) x_stage(s + 1);
+        __syncthreads();
+      }
+      if (active) {
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+          const R wi = (xP[i] - Xb[(k + 1) * NX + i]) * R(P.Pxinv[i]);
+          sm[L.w + k * NX + i] = wi;
+          dmax = rmax(dmax, fabs(wi));
+        }
+      }
+    } else if (role.kind == 'M') {  // the single columns, and what needs no integration
+      const int k = k0 + lane;
+      const bool active = lane < W && k < N - 1;
+      const R* st = sm + D.stage + (active ? lane : 0) * D.sa;
+      ColState<R> C[COL_SINGLES];
+#pragma unroll
+      for (int c = 0; c < COL_SINGLES; ++c)
+#pragma unroll
+        for (int i = 0; i < NX; ++i) C[c].P[i] = C[c].S[i] = (i == c) ? R(1) : R(0);
+      __syncthreads();
+#pragma unroll 1
+      for (int n = 0; n < nsub; ++n) {
+        if (active) singles_stage<R, NU, 0, 0>(C, st, h, h2, h6);
+        __syncthreads();
+        if (active) singles_stage<R, NU, 1, 0>(C, st + JS, h, h2, h6);
+        __syncthreads();
+        if (active) singles_stage<R, NU, 2, 0>(C, st, h, h2, h6);
+        __syncthreads();
+        if (active) singles_stage<R, NU, 3, 0>(C, st + JS, h, h2, h6);
+        __syncthreads();
+      }
+      if (active) {
+        singles_store<R, NU, 0>(P, L, sm, k, C);
+        R* Am = sm + L.Am + k * STM_SAS;
+        Am[stm_index(IY, IY)] = R(1) * R(P.Px[IY]) * R(P.Pxinv[IY]);
+        for (int q = kStm.nnz; q < STM_SAS; ++q) Am[q] = R(0);  // the block's zero and padding
+      }
+    } else if (role.kind == 'U') {  // control columns
+      const int t = role.index * 32 + lane, ci = t / W, k = k0 + t - ci * W;
+      const bool active = ci < 2 * NU && k < N - 1, minus = ci < NU;
+      const int cu = active ? (minus ? ci : ci - NU) : 0;
+      constexpr unsigned ALL = (1u << NX) - 1u;
+      ColState<R> C;
+      col_wave<R, NU, ALL, ALL, true>(C, -1, sm + D.stage + (active ? k - k0 : 0) * D.sa, nsub, h, active, minus, cu);
+      if (active) {
+        const R pc = R(P.Pu[cu]);
+        R* Bt = sm + (minus ? L.Bm : L.Bp) + k * b_stride(NU) + cu;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) Bt[i * NU] = C.P[i] * pc * R(P.Pxinv[i]);
+      }
+    } else if (role.kind != 'C' || !classes_wave<R, NU, 0>(P, L, sm, D, role.index, W, k0, h)) {  // no columns
+      for (int s = 0; s < 4 * nsub + 1; ++s) __syncthreads();
+    }
+    __syncthreads();  // the next wave overwrites the stage buffers
+  }
+  R v[1] = {dmax};
+  block_max_k<R, 1>(v, sm + D.red);
+  return v[0];
+}
+#endif
+
 // Sec. 2.3.2: hat eps_k, the dilation box, hat z_i (every component of
 // x_1 = (x0, 0) is fixed) and hat z_f (components selected by E_f).
 template <typename R, int NU>
