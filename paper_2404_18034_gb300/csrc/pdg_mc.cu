@@ -72,21 +72,26 @@ using namespace pdg;
 #endif
 // The fixed-point loop of FP64 instances runs 8 lanes a node (4 for NX <= 8):
 // internal variant 4 is built for up to 256 threads (N = 32), variant 5 for up
-// to 128 (N <= 16; 3-DoF N <= 32).  6-DoF takes two CTAs of 128 threads an SM
-// at 255 registers: three at 168 spill, are no faster on full batches (60.8
-// against 60.9 ms, 4096 instances, N = 15) and slower alone (7.6 against 7.1 ms,
-// 24 instances); four spill more (83 ms).  3-DoF's smaller tiles fit 168.
+// to 128 (N <= 16; 3-DoF N <= 32), variant 6 for up to 192 (N <= 24).
+// 6-DoF at 128 threads takes two CTAs an SM at 255 registers: three at 168
+// spill, are no faster on full batches (60.8 against 60.9 ms, 4096 instances,
+// N = 15) and slower alone (7.6 against 7.1 ms, 24 instances); four spill more
+// (83 ms).  3-DoF's smaller tiles fit 168.  At 160 and 192 threads 255 registers
+// leave one CTA an SM, 168 two: 17.3 against 22.2 us an iteration (1500
+// instances, N = 17), but 2.6 against 2.2 us where every instance has an SM
+// to itself.  At 256 threads two CTAs (128 registers) are slower, 20.6 against
+// 15.8 us (1024 instances, N = 30).
 #define PDG_FX_MAXT 256
-#define PDG_FX_MINB 1
-#define PDG_FX_MINB128 (pdg::NX <= 8 ? 3 : 2)
+#define PDG_FX_T(PV) ((PV) == 4 ? PDG_FX_MAXT : (PV) == 6 ? 192 : 128)
+#define PDG_FX_B(PV) ((PV) == 4 ? 1 : (PV) == 6 ? 2 : pdg::NX <= 8 ? 3 : 2)
 #define PDG_LB_PERS(R, PV)                                                                  \
-  __launch_bounds__((PV) >= 4 ? ((PV) == 4 ? PDG_FX_MAXT : 128) : (PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT  \
+  __launch_bounds__((PV) >= 4 ? PDG_FX_T(PV) : (PV) == 3 && sizeof(R) == 4 ? PDG_KS_PERS_MAXT  \
                     : ((PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512)), \
-                    (PV) >= 4 ? ((PV) == 4 ? PDG_FX_MINB : PDG_FX_MINB128) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
+                    (PV) >= 4 ? PDG_FX_B(PV) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 #define PDG_LB(R, PV)                                                                       \
-  __launch_bounds__((PV) >= 4 ? ((PV) == 4 ? PDG_FX_MAXT : 128)                               \
+  __launch_bounds__((PV) >= 4 ? PDG_FX_T(PV)                                                   \
                     : (PV) == 2 && sizeof(R) == 4 ? PDG_REG_MAXT_F32 : (sizeof(R) == 8 ? PDG_FP64_MAXT : 512), \
-                    (PV) >= 4 ? ((PV) == 4 ? PDG_FX_MINB : PDG_FX_MINB128) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
+                    (PV) >= 4 ? PDG_FX_B(PV) : sizeof(R) == 8 ? PDG_FP64_MINB : ((PV) == 1 ? PDG_FP32_MIN_BLOCKS : 1))
 
 namespace {
 
@@ -1011,7 +1016,7 @@ struct Plan {
   int Tr;  // threads of the other plain-form kernels
   int pv;  // 1 shared-memory PIPG, 2 register PIPG, 3 register tiles
   // the plain form's PIPG kernel: its threads, and its PIPG loop as the solve
-  // kernel's (kv): pv, or 4, 5 where form 1 runs in fixed point
+  // kernel's (kv): pv, or 4 to 6 where form 1 runs in fixed point
   int Tp, kp;
   int kv;
 };
@@ -1023,7 +1028,8 @@ static size_t solve_smem(int N, int nu, int T, int kv) {
   return (size_t)(kv >= 4 ? make_fx_lay(L).end : L.total) * sizeof(R);
 }
 
-static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bool use_override = true) {
+// B: instances of the launch (variant 6 is for batches of more than one an SM)
+static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* why, bool use_override = true) {
   const int treg = pipg_reg_threads(N, h->p.nu);
   const int maxt = h->p.precision == 1 ? PDG_REG_MAXT_F32 : 512;
   const int ov = use_override ? h->threads_override : 0;
@@ -1063,7 +1069,8 @@ static bool plan_for(const pdg_handle* h, int N, Plan* out, std::string* why, bo
     // the plain form's PIPG kernel runs no more threads than its lane groups
     // (3-DoF: 64 of the discretization's 128 at N = 15, so twice the CTAs)
     const int Tp = !fx ? T : (tks < 64 ? 64 : tks);
-    *out = {T, T, 1, Tp, !fx ? 1 : Tp <= 128 ? 5 : 4, !fx ? 1 : T <= 128 ? 5 : 4};
+    auto variant = [&](int t) { return t <= 128 ? 5 : (t <= 192 && B > h->num_sms ? 6 : 4); };
+    *out = {T, T, 1, Tp, !fx ? 1 : variant(Tp), !fx ? 1 : variant(T)};
   }
   return true;
 }
@@ -1079,14 +1086,14 @@ static PersistentFn<R, NU> persistent_fn(int pv, bool ck = false) {
     if (ck && pv == 1) return k_persistent<R, NU, 1, true>;
   }
   if constexpr (sizeof(R) == 8) {
-    if (pv >= 4) return pv == 5 ? k_persistent<R, NU, 5> : k_persistent<R, NU, 4>;
+    if (pv >= 4) return pv == 6 ? k_persistent<R, NU, 6> : pv == 5 ? k_persistent<R, NU, 5> : k_persistent<R, NU, 4>;
   }
   return pv == 3 ? k_persistent<R, NU, 3> : (pv == 2 ? k_persistent<R, NU, 2> : k_persistent<R, NU, 1>);
 }
 template <typename R, int NU>
 static PlainPipgFn<R, NU> plain_pipg_fn(int pv) {
   if constexpr (sizeof(R) == 8) {
-    if (pv >= 4) return pv == 5 ? k_plain_pipg<R, NU, 5> : k_plain_pipg<R, NU, 4>;
+    if (pv >= 4) return pv == 6 ? k_plain_pipg<R, NU, 6> : pv == 5 ? k_plain_pipg<R, NU, 5> : k_plain_pipg<R, NU, 4>;
   }
   return pv == 3 ? k_plain_pipg<R, NU, 3> : (pv == 2 ? k_plain_pipg<R, NU, 2> : k_plain_pipg<R, NU, 1>);
 }
@@ -1108,8 +1115,9 @@ struct Kern {
 #endif
     if constexpr (sizeof(R) == 8) {
       const void* fp64[] = {(const void*)k_persistent<R, NU, 1, true>, (const void*)k_persistent<R, NU, 4>,
-                            (const void*)k_persistent<R, NU, 5>, (const void*)k_plain_pipg<R, NU, 4>,
-                            (const void*)k_plain_pipg<R, NU, 5>};
+                            (const void*)k_persistent<R, NU, 5>, (const void*)k_persistent<R, NU, 6>,
+                            (const void*)k_plain_pipg<R, NU, 4>, (const void*)k_plain_pipg<R, NU, 5>,
+                            (const void*)k_plain_pipg<R, NU, 6>};
       for (const void* f : fp64) PDG_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     return 0;
@@ -1138,7 +1146,7 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
                      double* fuel, int* status, int* scp_iters, long long* pipg_iters, int* trace, cudaStream_t s) {
   Plan pl;
   std::string why;
-  if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T;
   const Lay L = make_lay(h->n_max, NU, T);
   // of the persistent kernel or the plain form's PIPG kernel, and of the plain form's others
@@ -1193,7 +1201,7 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
     PDG_CUDA(h, cudaEventRecord(h->ev_in, s));
     for (int N = h->n_max; N >= 2; --N) {
       Plan pn;
-      if (!plan_for(h, N, &pn, &why, N == h->n_max)) return fail(h, PDG_EINVAL, why);
+      if (!plan_for(h, B, N, &pn, &why, N == h->n_max)) return fail(h, PDG_EINVAL, why);
       const int Tn = pn.T;
       const PersistentFn<R, NU> kpn = persistent_fn<R, NU>(pn.kv);
       const Lay Ln = make_lay(N, NU, Tn);
@@ -1315,7 +1323,7 @@ static int run_subproblem(pdg_handle* h, int B, const double* x0, const int* Ns,
                           double* Am, double* Bm, double* Bp, double* w, cudaStream_t s) {
   Plan pl;
   std::string why;
-  if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.Tr;
   const Lay L = make_lay(h->n_max, NU, T);
   const size_t smem = (size_t)L.total * sizeof(R);
@@ -1331,7 +1339,7 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
                     double* step, int* iters, cudaStream_t s) {
   Plan pl;
   std::string why;
-  if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
   const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   h->last_variant = pl.pv;
@@ -1409,7 +1417,7 @@ static int run_noalloc(pdg_handle* h, int B, const double* x0, const int* Ns, do
                        double* fuel, int* status, int* scp_iters, long long* pipg_iters, cudaStream_t s) {
   Plan pl;
   std::string why;
-  if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
   const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   const Lay L = make_lay(h->n_max, NU, T);
@@ -1483,7 +1491,7 @@ static int run_grad(pdg_handle* h, int B, const double* x0, const int* Ns, const
   // otherwise k_grad reruns that loop forward and writes the checkpoints.
   Plan pl;
   std::string why;
-  if (!plan_for(h, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
   const bool ckrec = pl.pv == 1;
   const int rec_stride = h->n_max * (NX + NU) + (Lg.img - Lg.xh) + 2 +
                          (ckrec ? h->n_max * (NX + NU) + nck_max * ss : 0);
