@@ -1486,13 +1486,15 @@ static int run_grad(pdg_handle* h, int B, const double* x0, const int* Ns, const
   if (h->p.rk4_substeps > 32) return fail(h, PDG_EINVAL, "gradients support at most 32 RK4 substeps");
   const int ss = Ag.ss;
   const int nck_max = (h->p.pipg_jmax + 49) / 50;
-  // With the shared-memory PIPG form the solve itself records the last PIPG
-  // loop's checkpoints and final iterate (k_persistent's CK instantiation);
-  // otherwise k_grad reruns that loop forward and writes the checkpoints.
+  // A solve whose PIPG loop runs in FP64 in shared memory records the last
+  // loop's checkpoints and final iterate itself (k_persistent's CK
+  // instantiation).  Otherwise k_grad reruns that loop forward and writes the
+  // checkpoints: behind a solve in fixed point too, whose other loops (about
+  // eight) take a third of the FP64 loop's time.
   Plan pl;
   std::string why;
   if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
-  const bool ckrec = pl.pv == 1;
+  const bool ckrec = pl.kv == 1;
   const int rec_stride = h->n_max * (NX + NU) + (Lg.img - Lg.xh) + 2 +
                          (ckrec ? h->n_max * (NX + NU) + nck_max * ss : 0);
   // per instance: [checkpoints of the state every 50 iterations,] one segment's records
