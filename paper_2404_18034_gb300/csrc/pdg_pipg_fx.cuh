@@ -22,9 +22,11 @@ namespace pdg {
 // an iterate is split as h 2^31 + 2 l; h h, h l and l h are summed in two
 // 64-bit accumulators, which 8 terms cannot overflow, and l l (below half of
 // the last unit) is left out.  Against 80-bit arithmetic on the subproblems of
-// 6-DoF and 3-DoF solves (2000 iterations) the results are as near as the
-// FP64 loop's: x_hat 0.5 to 1 times its error, u_hat and phi 0.5 to 2 times,
-// all within 2e-15.
+// 6-DoF and 3-DoF solves (2000 iterations), with the FP64 loop's errors in
+// brackets: first SCP iterations x_hat 1 to 8e-16 (1 to 2e-15), u_hat 1 to
+// 3e-16 (2 to 4e-16), phi 1 to 3e-16 (3 to 6e-16); later ones, whose iterates
+// are small, x_hat 0.4 to 3.5e-15 (0.4 to 6e-15), u_hat 0.4 to 1.5e-15 (0.2 to
+// 1e-15), phi 0.1 to 1.4e-15 (0.1 to 0.8e-15).
 //
 // Range.  Every iterate that is multiplied or stored is or-ed into a word of
 // magnitudes; every 10 iterations the CTA looks at it.  A value beyond the
