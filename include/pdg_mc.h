@@ -251,7 +251,11 @@ int pdg_mc_autotune(pdg_handle* h, int B, const double* x0, const int* n_nodes, 
 /* Choose how the PIPG loop (Alg. PIPG_custom, Sec. 3) is laid out on the
  * CTA.  Results agree to rounding; only speed differs.
  *   form 1: blocks hat A^-, hat B^+- and the iterates in shared memory, any
- *           thread count (one thread per block row or column, looped);
+ *           thread count (one thread per block row or column, looped).  In
+ *           FP64 the loop runs in 64-bit fixed point on form 3's lane groups
+ *           where the thread count lies in [round32(8 N), 256] (4 N when
+ *           NX <= 8), soc_thrust is off and the data suits, with errors of
+ *           the size of FP64 rounding; in FP64 otherwise;
  *   form 2: every thread keeps its block rows/columns and iterate entries in
  *           registers for the whole loop; only the vectors exchanged between
  *           the primal and dual steps go through shared memory.  Needs
