@@ -363,28 +363,8 @@ k_plain_init(const DParams P, int B, int Nmax, const double* __restrict__ x0, co
   if (threadIdx.x == 0) W.st[b] = ST_RUNNING;
 }
 
-template <typename R, int NU>
-__global__ void __launch_bounds__(512, sizeof(R) == 4 ? PDG_FP32_DISC_MIN_BLOCKS : 1)
-k_plain_disc(const DParams P, int B, int Nmax, const int* __restrict__ Ns, PlainWs W) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  R* sm = reinterpret_cast<R*>(smraw);
-  const int b = blockIdx.x;
-  if (W.st[b] != ST_RUNNING) return;
-  if (plain_aborted(P)) return;  // k_plain_update ends the instance
-  const int N = Ns ? Ns[b] : Nmax;
-  const Lay L = make_lay(N, NU, blockDim.x);
-  R* img = reinterpret_cast<R*>(W.img) + (size_t)b * W.istride;
-  copy_g2s(sm + L.x0, img + L.x0, L.Am - L.x0);  // x0, Xb, Ub
-  __syncthreads();
-  const R defect = phase_discretize<R, NU>(P, L, sm);
-  phase_scale_extra<R, NU>(P, L, sm);
-  __syncthreads();
-  copy_s2g(img + L.Am, sm + L.Am, L.xh - L.Am);  // Am .. zf
-  if (threadIdx.x == 0) img[L.sc + 1] = defect;
-}
-
 #ifdef PDG_MODEL_HAS_COLUMN_CLASSES
-// The same by column classes (discretize_cols), for models that declare them;
+// The discretization by column classes (discretize_cols), for models that declare them;
 // built for up to MAXT threads.  Two CTAs an SM: one is slower (18.6 against
 // 17.5 ms for an SCP iteration with 20 PIPG iterations, 4096 instances, N = 15;
 // FP32, 16384 instances: 9.3 against 6.3), three are no faster.
@@ -403,6 +383,26 @@ k_plain_disc_cols(const DParams P, int B, int Nmax, const int* __restrict__ Ns, 
   copy_g2s(sm + L.x0, img + L.x0, L.Am - L.x0);  // x0, Xb, Ub
   __syncthreads();
   const R defect = discretize_cols<R, NU>(P, L, sm, D);
+  phase_scale_extra<R, NU>(P, L, sm);
+  __syncthreads();
+  copy_s2g(img + L.Am, sm + L.Am, L.xh - L.Am);  // Am .. zf
+  if (threadIdx.x == 0) img[L.sc + 1] = defect;
+}
+#else
+template <typename R, int NU>
+__global__ void __launch_bounds__(512, sizeof(R) == 4 ? PDG_FP32_DISC_MIN_BLOCKS : 1)
+k_plain_disc(const DParams P, int B, int Nmax, const int* __restrict__ Ns, PlainWs W) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  R* sm = reinterpret_cast<R*>(smraw);
+  const int b = blockIdx.x;
+  if (W.st[b] != ST_RUNNING) return;
+  if (plain_aborted(P)) return;  // k_plain_update ends the instance
+  const int N = Ns ? Ns[b] : Nmax;
+  const Lay L = make_lay(N, NU, blockDim.x);
+  R* img = reinterpret_cast<R*>(W.img) + (size_t)b * W.istride;
+  copy_g2s(sm + L.x0, img + L.x0, L.Am - L.x0);  // x0, Xb, Ub
+  __syncthreads();
+  const R defect = phase_discretize<R, NU>(P, L, sm);
   phase_scale_extra<R, NU>(P, L, sm);
   __syncthreads();
   copy_s2g(img + L.Am, sm + L.Am, L.xh - L.Am);  // Am .. zf
@@ -1102,7 +1102,10 @@ struct Kern {
   static int prepare(pdg_handle* h, int threads, size_t smem) {
     const void* fns[] = {(const void*)k_persistent<R, NU, 1>, (const void*)k_persistent<R, NU, 2>,
                          (const void*)k_persistent<R, NU, 3>, (const void*)k_plain_init<R, NU>,
-                         (const void*)k_plain_disc<R, NU>, (const void*)k_plain_power<R, NU>,
+#ifndef PDG_MODEL_HAS_COLUMN_CLASSES
+                         (const void*)k_plain_disc<R, NU>,
+#endif
+                         (const void*)k_plain_power<R, NU>,
                          (const void*)k_plain_pipg<R, NU, 1>, (const void*)k_plain_pipg<R, NU, 2>,
                          (const void*)k_plain_pipg<R, NU, 3>, (const void*)k_plain_update<R, NU>,
                          (const void*)k_subproblem<R, NU>};

@@ -42,7 +42,7 @@ namespace pdg {
 // (4096 instances, N = 15): 30.1 ms per 1000 iterations, 2330 cycles an
 // instance and iteration against 6890 of phase_pipg; N = 30 (1024 instances)
 // 15.9 ms.  Bound by latency and issue: two CTAs (8 warps) an SM at 255
-// registers, 1.5 instructions a clock; a third CTA at 168 registers adds
+// registers, 1.4 instructions a clock; a third CTA at 168 registers adds
 // spills and no speed.
 // ---------------------------------------------------------------------------
 struct FxM { int h, l; };  // matrix entry: (h 2^30 + l) 2^-60
