@@ -129,7 +129,8 @@ __device__ __forceinline__ unsigned block_or(unsigned v, unsigned* red) {
 // mass and velocity), they take the even places, and a quarter of every
 // lane's tile, even rows times odd columns, is structurally zero: it is
 // neither held nor multiplied (16 of 96 tile registers, 48 of 288
-// multiply-adds).  Other models keep their order and the whole tile.
+// multiply-adds).  Other models, and those with fewer states than half of the
+// places, keep their order and the whole tile.
 struct FxOrder {
   unsigned char state[KS_NXB], place[KS_NXB];  // state NX and up: padding
   bool split;
@@ -138,9 +139,9 @@ __host__ __device__ constexpr FxOrder make_fx_order() {
   FxOrder F{};
   const StmOrder S = make_stm_order();
   unsigned even = 0;
-  for (int a = 0; a < KS_NXB / 2; ++a) even |= 1u << S.row_order[NX - 1 - a];  // the sparsest rows
-  F.split = true;
-  for (int a = 0; a < KS_NXB / 2; ++a) F.split = F.split && (S.row_mask[S.row_order[NX - 1 - a]] & ~even) == 0;
+  F.split = NX >= KS_NXB / 2;
+  for (int a = 0; F.split && a < KS_NXB / 2; ++a) even |= 1u << S.row_order[NX - 1 - a];  // the sparsest rows
+  for (int a = 0; F.split && a < KS_NXB / 2; ++a) F.split = (S.row_mask[S.row_order[NX - 1 - a]] & ~even) == 0;
   int e = 0, o = 1;
   for (int i = 0; i < KS_NXB; ++i) {
     int p = i;
