@@ -1156,7 +1156,24 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
   const size_t smem_r = (size_t)plain_total(h->n_max, NU, pl.Tp, pl.Tr) * sizeof(R);
   if (L.ipw < 1 || make_lay(h->n_max, NU, pl.Tr).ipw < 1)
     return fail(h, PDG_EINVAL, "threads per CTA too small for one discretization interval");
-  if (int rc = Kern<R, NU>::prepare(h, T, smem > smem_r ? smem : smem_r)) return rc;
+  // Shape classes: every class is planned before the kernels' shared-memory
+  // limit is set, since a smaller class can ask for more than n_max does (a
+  // thread setting counts for n_max alone, the others choose their own loop).
+  Plan pn[NMAX + 1];
+  int occ_n[NMAX + 1] = {};
+  size_t smem_n[NMAX + 1] = {}, smem_max = smem > smem_r ? smem : smem_r;
+  const bool classes = mode == 2 && Ns;
+  for (int N = 2; classes && N <= h->n_max; ++N) {
+    if (!plan_for(h, B, N, &pn[N], &why, N == h->n_max)) return fail(h, PDG_EINVAL, why);
+    smem_n[N] = solve_smem<R>(N, NU, pn[N].T, pn[N].kv);
+    if (smem_n[N] > smem_max) smem_max = smem_n[N];
+  }
+  if (int rc = Kern<R, NU>::prepare(h, T, smem_max)) return rc;
+  for (int N = 2; classes && N <= h->n_max; ++N) {
+    PDG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_n[N], persistent_fn<R, NU>(pn[N].kv), pn[N].T,
+                                                              smem_n[N]));
+    if (occ_n[N] < 1) return fail(h, PDG_EINVAL, "a shape class does not fit on an SM");
+  }
   const PersistentFn<R, NU> kp = persistent_fn<R, NU>(pl.kv, h->ck_rec && mode == 1);
   int occ = 0;
   PDG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, T, smem));
@@ -1202,16 +1219,9 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
     PDG_CUDA(h, cudaGetLastError());
     PDG_CUDA(h, cudaEventRecord(h->ev_in, s));
     for (int N = h->n_max; N >= 2; --N) {
-      Plan pn;
-      if (!plan_for(h, B, N, &pn, &why, N == h->n_max)) return fail(h, PDG_EINVAL, why);
-      const int Tn = pn.T;
-      const PersistentFn<R, NU> kpn = persistent_fn<R, NU>(pn.kv);
-      const Lay Ln = make_lay(N, NU, Tn);
-      const size_t smem_n = solve_smem<R>(N, NU, Tn, pn.kv);
-      if (Ln.ipw < 1) continue;
-      int occ_n = 0;
-      PDG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_n, kpn, Tn, smem_n));
-      if (occ_n < 1) return fail(h, PDG_EINVAL, "a shape class does not fit on an SM");
+      const int Tn = pn[N].T;
+      const PersistentFn<R, NU> kpn = persistent_fn<R, NU>(pn[N].kv);
+      if (make_lay(N, NU, Tn).ipw < 1) continue;
       cudaStream_t cs = h->cls_streams[N];
       if (!cs) {
         PDG_CUDA(h, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -1219,8 +1229,8 @@ static int run_solve(pdg_handle* h, int B, const double* x0, const int* Ns, int 
         PDG_CUDA(h, cudaEventCreateWithFlags(&h->cls_events[N], cudaEventDisableTiming));
       }
       PDG_CUDA(h, cudaStreamWaitEvent(cs, h->ev_in, 0));
-      const int grid = (int)((long long)occ_n * h->num_sms < B ? (long long)occ_n * h->num_sms : B);
-      kpn<<<grid, Tn, smem_n, cs>>>(h->dp, B, h->n_max, x0, Ns, X, U, tf, fuel, status, scp_iters, pipg_iters, trace,
+      const int grid = (int)((long long)occ_n[N] * h->num_sms < B ? (long long)occ_n[N] * h->num_sms : B);
+      kpn<<<grid, Tn, smem_n[N], cs>>>(h->dp, B, h->n_max, x0, Ns, X, U, tf, fuel, status, scp_iters, pipg_iters, trace,
                                     queues + N, h->rec_ptr, h->rec_stride, perm, class_off, N);
       PDG_CUDA(h, cudaGetLastError());
       PDG_CUDA(h, cudaEventRecord(h->cls_events[N], cs));
