@@ -255,7 +255,8 @@ int pdg_mc_autotune(pdg_handle* h, int B, const double* x0, const int* n_nodes, 
  *           FP64 the loop runs in 64-bit fixed point on form 3's lane groups
  *           where the thread count lies in [round32(8 N), 256] (4 N when
  *           NX <= 8), soc_thrust is off and the data suits, with errors of
- *           the size of FP64 rounding; in FP64 otherwise;
+ *           the size of FP64 rounding; in FP64 otherwise (so that a thread
+ *           setting outside that range, e.g. 288, asks for the FP64 loop);
  *   form 2: every thread keeps its block rows/columns and iterate entries in
  *           registers for the whole loop; only the vectors exchanged between
  *           the primal and dual steps go through shared memory.  Needs
@@ -275,6 +276,13 @@ int pdg_mc_set_pipg_form(pdg_handle* h, int form);
 /* The PIPG form (1, 2 or 3) of the handle's last solve or SCP step, 0 before
  * the first; PDG_EINVAL for a NULL handle. */
 int pdg_mc_pipg_form(const pdg_handle* h);
+
+/* How the handle's PIPG loops of form 1 in FP64 ran since pdg_mc_init, where
+ * the launch chose the fixed-point loop (see pdg_mc_set_pipg_form): loops that
+ * finished in fixed point, the times that part of one was run again at a
+ * coarser unit, and loops whose data did not suit and that ran in FP64.  Each
+ * pointer may be NULL.  Synchronizes the device. */
+int pdg_mc_pipg_loops(pdg_handle* h, long long* fixed_point, long long* again, long long* fp64);
 
 /* Solve without allocating: for callers that cannot call cudaMalloc while
  * they run, e.g. code inside a region that a memory pool or allocator owns,

@@ -37,6 +37,8 @@ struct DParams {
   double mp[16];     // constants of a model supplied through PDG_MODEL_HEADER
   const int* abort_flag;  // the handle's abort word (host memory mapped into the
                           // device's address space), or null
+  unsigned long long* loops;  // the handle's counts of PIPG loops (device memory): finished in
+                              // fixed point, parts of them run again, handed to the FP64 loop
 };
 
 // The handle's abort request, read at system scope so that a store from a

@@ -106,7 +106,12 @@ template <typename R, int NU, int PV, bool CK = false>
 __device__ __forceinline__ int run_pipg(const DParams& P, const Lay& L, R* sm, R sigma, int force,
                                         double* ck = nullptr) {
   if constexpr (PV >= 4) {
-    const int it = phase_pipg_fx<NU>(P, L, sigma, force);
+    int again = 0;
+    const int it = phase_pipg_fx<NU>(P, L, sigma, force, &again);
+    if (threadIdx.x == 0) {
+      atomicAdd(P.loops + (it >= 0 ? 0 : 2), 1ull);
+      if (again > 0) atomicAdd(P.loops + 1, (unsigned long long)again);
+    }
     return it >= 0 ? it : pipg_fp64<NU>(P, L, sm, sigma, force);
   } else if constexpr (PV == 2) return phase_pipg_reg<R, NU>(P, L, sm, sigma, force);
   else if constexpr (PV == 3) return phase_pipg_ks<R, NU>(P, L, sm, sigma, force);
@@ -1595,6 +1600,15 @@ int pdg_mc_init(const pdg_params* p, int n_max, pdg_handle** out) {
       return PDG_ECUDA;
     }
     h->dp.abort_flag = static_cast<const int*>(dptr);
+    ea = cudaMalloc((void**)&h->dp.loops, 3 * sizeof(unsigned long long));
+    if (ea == cudaSuccess) ea = cudaMemset(h->dp.loops, 0, 3 * sizeof(unsigned long long));
+    if (ea != cudaSuccess) {
+      if (h->dp.loops) cudaFree(h->dp.loops);
+      cudaFreeHost(h->abort_host);
+      delete h;
+      g_init_err = std::string("counts of PIPG loops: ") + cudaGetErrorString(ea);
+      return PDG_ECUDA;
+    }
   }
   *out = h;
   g_init_err.clear();
@@ -1604,6 +1618,7 @@ int pdg_mc_init(const pdg_params* p, int n_max, pdg_handle** out) {
 void pdg_mc_destroy(pdg_handle* h) {
   if (!h) return;
   cudaDeviceSynchronize();
+  if (h->dp.loops) cudaFree(h->dp.loops);
   if (h->img) cudaFree(h->img);
   if (h->ints) cudaFree(h->ints);
   if (h->lit) cudaFree(h->lit);
@@ -1744,6 +1759,19 @@ int pdg_mc_set_pipg_form(pdg_handle* h, int form) {
 }
 
 int pdg_mc_pipg_form(const pdg_handle* h) { return h ? h->last_variant : PDG_EINVAL; }
+
+int pdg_mc_pipg_loops(pdg_handle* h, long long* fixed_point, long long* again, long long* fp64) {
+  if (!h) return PDG_EINVAL;
+  h->err.clear();
+  PDG_CUDA(h, cudaSetDevice(h->device));
+  PDG_CUDA(h, cudaDeviceSynchronize());
+  unsigned long long n[3];
+  PDG_CUDA(h, cudaMemcpy(n, h->dp.loops, sizeof n, cudaMemcpyDeviceToHost));
+  if (fixed_point) *fixed_point = (long long)n[0];
+  if (again) *again = (long long)n[1];
+  if (fp64) *fp64 = (long long)n[2];
+  return PDG_OK;
+}
 
 int pdg_mc_autotune(pdg_handle* h, int B, const double* x0, const int* n_nodes, int mode, int* threads_out,
                     int* form_out, double* solves_per_s, void* cuda_stream) {

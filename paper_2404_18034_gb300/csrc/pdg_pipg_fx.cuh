@@ -195,9 +195,10 @@ __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
 // iterations between two looks at the magnitudes
 constexpr int FX_WINDOW = 10;
 
-// Returns the iterations run (at least one), or -1 with the image untouched.
+// Returns the iterations run (at least one), or -1 with the image untouched;
+// *again the restarts at a coarser unit.
 template <int NU>
-__device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, double sigma, int force) {
+__device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, double sigma, int force, int* again) {
   using U = unsigned long long;
   extern __shared__ __align__(16) unsigned char smraw[];
   double* const sm = reinterpret_cast<double*>(smraw);
@@ -665,7 +666,10 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         __syncthreads();
       }
     }
-    if (over) continue;
+    if (over) {
+      ++*again;
+      continue;
+    }
     // the unextrapolated iterates to the image (warm start of the next SCP iteration)
     const double un = ldexp(1.0, gb - 61);
     __syncthreads();

@@ -26,7 +26,8 @@ EXPORTS = ("pdg_mc_init", "pdg_mc_destroy", "pdg_mc_last_error", "pdg_mc_solve_b
            "pdg_mc_solve_batch_host", "pdg_mc_subproblem", "pdg_mc_scp_step", "pdg_mc_launch_info",
            "pdg_mc_set_threads", "pdg_mc_probe_fma", "pdg_mc_solve_batch_noalloc",
            "pdg_mc_grad_batch", "pdg_mc_set_pipg_form", "pdg_mc_pipg_form", "pdg_mc_probe_fma_lanes",
-           "pdg_mc_autotune", "pdg_mc_model_nx", "pdg_mc_abort", "pdg_mc_clear_abort")
+           "pdg_mc_autotune", "pdg_mc_model_nx", "pdg_mc_abort", "pdg_mc_clear_abort",
+           "pdg_mc_pipg_loops")
 
 
 class PdgParams(C.Structure):
@@ -101,12 +102,13 @@ def load_library(path: Optional[str] = None, model: str = "6dof"):
     L.pdg_mc_autotune.argtypes = [_VP, C.c_int, _VP, _VP, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int),
                                   C.POINTER(C.c_double), _VP]
     L.pdg_mc_pipg_form.argtypes = [_VP]
+    L.pdg_mc_pipg_loops.argtypes = [_VP] + [C.POINTER(C.c_longlong)] * 3
     L.pdg_mc_abort.argtypes = [_VP]
     L.pdg_mc_clear_abort.argtypes = [_VP]
     for name in ("pdg_mc_init", "pdg_mc_solve_batch", "pdg_mc_solve_batch_host", "pdg_mc_subproblem",
                  "pdg_mc_scp_step", "pdg_mc_launch_info", "pdg_mc_set_threads", "pdg_mc_probe_fma",
                  "pdg_mc_solve_batch_noalloc", "pdg_mc_grad_batch", "pdg_mc_set_pipg_form", "pdg_mc_pipg_form",
-                 "pdg_mc_probe_fma_lanes", "pdg_mc_autotune", "pdg_mc_abort", "pdg_mc_clear_abort"):
+                 "pdg_mc_probe_fma_lanes", "pdg_mc_autotune", "pdg_mc_abort", "pdg_mc_clear_abort", "pdg_mc_pipg_loops"):
         getattr(L, name).restype = C.c_int
     _libs[(path, model)] = L
     return L
@@ -333,6 +335,12 @@ class Solver:
         self._check(self.lib.pdg_mc_launch_info(self.h, C.byref(t), C.byref(c), C.byref(s)), "pdg_mc_launch_info")
         return dict(threads=t.value, ctas_per_sm=c.value, smem_bytes=s.value,
                     pipg_form=int(self.lib.pdg_mc_pipg_form(self.h)))
+
+    def pipg_loops(self):
+        """pdg_mc_pipg_loops: how the handle's fixed-point PIPG loops ran so far."""
+        n = [C.c_longlong() for _ in range(3)]
+        self._check(self.lib.pdg_mc_pipg_loops(self.h, *[C.byref(v) for v in n]), "pdg_mc_pipg_loops")
+        return dict(fixed_point=n[0].value, again=n[1].value, fp64=n[2].value)
 
     def autotune(self, x0, n_nodes=None, mode: int = 1, stream=None):
         """pdg_mc_autotune on a device batch: returns (threads, form,
