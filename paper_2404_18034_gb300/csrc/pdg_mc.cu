@@ -102,16 +102,21 @@ __device__ __noinline__ int pipg_fp64(const DParams& P, const Lay& L, double* sm
   return phase_pipg<double, NU>(P, L, sm, sigma, force);
 }
 
-template <typename R, int NU, int PV, bool CK = false>
+// The fixed-point loop out of line, for the persistent kernel: inside that
+// kernel's loops its invariants are hoisted and its registers spilled.
+template <int NU, int PV>
+__device__ __noinline__ int pipg_fx(const DParams& P, int nodes, double sigma, int force) {
+  return phase_pipg_fx<NU>(P, nodes, sigma, force);
+}
+
+template <typename R, int NU, int PV, bool CK = false, bool PERS = false>
 __device__ __forceinline__ int run_pipg(const DParams& P, const Lay& L, R* sm, R sigma, int force,
                                         double* ck = nullptr) {
   if constexpr (PV >= 4) {
-    int again = 0;
-    const int it = phase_pipg_fx<NU>(P, L, sigma, force, &again);
-    if (threadIdx.x == 0) {
-      atomicAdd(P.loops + (it >= 0 ? 0 : 2), 1ull);
-      if (again > 0) atomicAdd(P.loops + 1, (unsigned long long)again);
-    }
+    int it;
+    if constexpr (PERS) it = pipg_fx<NU, PV>(P, L.N, sigma, force);
+    else it = phase_pipg_fx<NU>(P, L.N, sigma, force);
+    if (threadIdx.x == 0) atomicAdd(P.loops + (it >= 0 ? 0 : 2), 1ull);
     return it >= 0 ? it : pipg_fp64<NU>(P, L, sm, sigma, force);
   } else if constexpr (PV == 2) return phase_pipg_reg<R, NU>(P, L, sm, sigma, force);
   else if constexpr (PV == 3) return phase_pipg_ks<R, NU>(P, L, sm, sigma, force);
@@ -270,12 +275,12 @@ k_persistent(const DParams P, int B, int Nmax, const double* __restrict__ x0, co
         if constexpr (CK) {
           const int ow = L.N * (NX + NU), nw = L.img - L.xh;
           double* ckp = rec + (size_t)C.b * rec_stride + ow + nw + 2 + ow;
-          jit = run_pipg<R, NU, PV, true>(P, L, sm, sigma, 0, ckp);
+          jit = run_pipg<R, NU, PV, true, true>(P, L, sm, sigma, 0, ckp);
           double* rf = rec + (size_t)C.b * rec_stride + ow + nw + 2;
           for (int t = threadIdx.x; t < ow; t += blockDim.x)
             rf[t] = double(t < L.N * NX ? sm[L.xh + t] : sm[L.uh + t - L.N * NX]);
         } else {
-          jit = run_pipg<R, NU, PV>(P, L, sm, sigma, 0);
+          jit = run_pipg<R, NU, PV, false, true>(P, L, sm, sigma, 0);
         }
       }
       const int bb = C.b;
@@ -1011,9 +1016,9 @@ static int threads_for(int N, int nu, int precision) {
 // PIPG form and CTA size for instances of up to N nodes.  Auto (variant 0):
 // FP32 takes the tiled register form (form 3; the shared-memory form is bound
 // by shared-memory bandwidth, form 2 by its operand loads), FP64 the
-// shared-memory form, whose loop then runs in 64-bit fixed point where it can.  In auto mode a thread-count override outside
-// what form 3 accepts selects the shared form; with form 2 or 3 requested it
-// is an error.
+// shared-memory form, whose loop then runs in 64-bit fixed point where it can.
+// In auto mode a thread-count override outside what form 3 accepts selects the
+// shared form; with form 2 or 3 requested it is an error.
 // The non-PIPG kernels of the plain form run with at most 512 threads.
 struct Plan {
   int T;   // threads of the solve kernel
@@ -1061,12 +1066,14 @@ static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* 
     *out = {T, T < 128 ? 128 : T, 3, T, 3, 3};
   } else {
     // FP64 runs the loop in 64-bit fixed point (phase_pipg_fx: about three times
-    // the FP64 loop's rate: 2330 against 6890 cycles an instance and iteration at N = 15) wherever its lane groups and its
-    // exchange region fit; not with the thrust projection, whose square roots
-    // are FP64 work, nor in the gradient's solve, which records FP64 states
+    // the FP64 loop's rate: 2330 against 6890 cycles an instance and iteration
+    // at N = 15) wherever its lane groups and its exchange region fit; not on
+    // fewer than FX_NMIN nodes (see there), not with the thrust projection, whose
+    // square roots are FP64 work, nor in a gradient's solve that records FP64
+    // states
     int T = ov > 0 ? ov : threads_for(N, h->p.nu, h->p.precision);
     if (T > 512) { *why = "the shared-memory PIPG form runs at most 512 threads per CTA"; return false; }
-    bool fx = h->p.precision == 0 && !h->p.soc_thrust && !h->ck_rec;
+    bool fx = h->p.precision == 0 && !h->p.soc_thrust && !h->ck_rec && N >= FX_NMIN;
     if (fx && ov == 0) T = T < tks ? tks : (T > PDG_FX_MAXT ? PDG_FX_MAXT : T);
     fx = fx && T >= tks && T <= PDG_FX_MAXT && solve_smem<double>(N, h->p.nu, T, 4) <= 226 * 1024;
     if (!fx && ov == 0) T = threads_for(N, h->p.nu, h->p.precision);

@@ -8,33 +8,55 @@ namespace pdg {
 // 32 x 32 + 64-bit integer multiply-adds (measured: 0.052 and 1.93 warp
 // instructions a clock and SM), so the FP64 loop of phase_pipg is bound by
 // the FP64 pipe, where three integer multiply-adds in place of one FMA cost a
-// twelfth.  This loop has no floating-point instruction in it.
+// twelfth.  The iteration here has no floating-point instruction in it; the
+// stop test compares in FP64.
 //
 // Variables.  With psi = phi / sqrt(omega), theta likewise, gamma = alpha
 // sqrt(omega) and M = gamma K, the iteration of Alg. PIPG_custom reads
 //   x' = c1 x~ - M^T psi~ + ...,  psi' = psi~ + M (2 x' - x~) + gamma (w + ...)
 // so one matrix M of spectral norm at most one serves both steps (x and u are
-// held negated: the primal step then only adds), and every iterate lives at one scale: 64-bit integers X in units of 2^(gb - 61) with
-// |X| < 2^61, gb chosen so that the largest iterate keeps one or two bits of
-// headroom (see rescaling below).
+// held negated: the primal step then only adds), and every iterate lives at
+// one scale: 64-bit integers X in units of 2^(gb - 61) with |X| < 2^61.
 //
 // Products.  M is held as h 2^30 + l in units of 2^-60 (both signed, 32 bits),
 // an iterate is split as h 2^31 + 2 l; h h, h l and l h are summed in two
-// 64-bit accumulators, which 8 terms cannot overflow, and l l (below half of
-// the last unit) is left out.  Against 80-bit arithmetic on the subproblems of
-// 6-DoF and 3-DoF solves (2000 iterations), with the FP64 loop's errors in
-// brackets: first SCP iterations x_hat 1 to 8e-16 (1 to 2e-15), u_hat 1 to
-// 3e-16 (2 to 4e-16), phi 1 to 3e-16 (3 to 6e-16); later ones, whose iterates
-// are small, x_hat 0.4 to 3.5e-15 (0.4 to 6e-15), u_hat 0.4 to 1.5e-15 (0.2 to
-// 1e-15), phi 0.1 to 1.4e-15 (0.1 to 0.8e-15).
+// 64-bit accumulators, and l l (below half of the last unit) is left out.
 //
 // Range.  Every iterate that is multiplied or stored is or-ed into a word of
-// magnitudes; every 10 iterations the CTA looks at it.  A value beyond the
-// range restarts the loop at a coarser unit from the warm start, which stays
-// in the image until the loop ends; where that does not help (or the data is
-// not finite, or |M| is not small because sigma was underestimated), -1 is
-// returned and the caller runs the FP64 loop.  Otherwise the unit follows the
-// largest iterate by shifts.
+// magnitudes; every 10 iterations the CTA looks at it.  The unit follows the
+// largest iterate by shifts, so that it fills the range (from a cold start it
+// keeps a bit or two of headroom while the iterates grow).  A value beyond the
+// range sends the loop back to the last look's state, ten iterations, at a unit
+// four times as coarse: that costs less than headroom would in precision.
+//
+// Precision.  The rounding is absolute, about 2^-60 of the range a sum, where
+// FP64's is 2^-53 of each entry: finer for whatever is within 2^-7 of the
+// largest iterate, and for small entries that large ones feed (their sums
+// round in FP64 at the large ones' scale).  What it could cost are groups that
+// sink far below the rest, so the loop returns -1, and the caller runs the
+// FP64 loop, where at the end the largest control or the largest phi is below
+// 2^-8 of the range, or theta, if any is not zero, below 2^-20 of it or weighed
+// against an eps below 2^-20 of it; and before the loop where a control column
+// has no entry of M of 2^-12 (with a gamma below 2^-24 the controls hardly move).
+// Default parameters stay within 2^-6.9, 2^-4 and 2^-8.7 (controls, phi,
+// columns), and theta sends about one in 10 000 of their loops to FP64.
+// Likewise where the data is not finite, an entry of M above 1.2 shows that the
+// power iteration fell short, or the iterates grow 2^40 past the data.
+//
+// Errors against 80-bit arithmetic in x_hat, u_hat, phi and theta, relative to
+// each array's largest, root mean square over the subproblems of SCP iterations
+// 1 to 9 of dispersed solves with N = 6 to 32 (1344, 768 and 768 of them; the
+// FP64 loop's in brackets; emulated on the host):
+//   6-DoF nu = 4    20   2.7e-16 (2.2e-15)  3.0e-16 (8.0e-16)  1.4e-16 (2.6e-16)  4.9e-15 (8.1e-15)
+//                  200   5.1e-16 (5.6e-15)  5.0e-16 (4.5e-15)  1.6e-16 (1.6e-15)  1.8e-15 (2.9e-15)
+//                 2000   3.7e-15 (4.6e-14)  3.1e-15 (4.0e-14)  6.3e-16 (1.6e-14)  6.3e-15 (3.0e-14)
+//   6-DoF nu = 7    20   6.5e-16 (5.2e-15)  6.8e-16 (7.9e-16)  2.2e-16 (2.4e-16)  1.0e-15 (2.1e-15)
+//                 2000   8.9e-16 (8.6e-15)  5.8e-16 (1.7e-15)  3.6e-16 (1.5e-15)  1.8e-14 (1.4e-14)
+//   3-DoF           20   9.8e-16 (1.1e-14)  3.6e-16 (6.1e-16)  1.3e-16 (2.3e-16)  3.4e-16 (2.8e-15)
+//                 2000   9.8e-16 (1.3e-14)  4.3e-16 (8.1e-16)  1.7e-16 (5.6e-16)  5.0e-16 (2.2e-15)
+// The virtual controls (w_ep 0.3 to 100): 1.0 to 8.4e-16 (3.6e-16 to 1.3e-14).
+// What stays behind are thetas far below phi: one in a thousand by about 5
+// times, more where P_x takes y far from the other states.
 //
 // Work split: the tiles and butterflies of phase_pipg_ks.  At N = 15 a CTA
 // runs 128 threads and about 4200 warp instructions an iteration, 900 of them
@@ -163,8 +185,14 @@ __host__ __device__ constexpr bool fx_zero(int s, int q) { return FX_SPLIT && (s
 // or node [N][KS_NXB], 2 u - u~ (split) and the control gradients [N][nup],
 // gamma theta~, gamma eps [N], the dilation box and, behind it, no box [N + 1], the fixed components of the
 // first and the last node [2][KS_NXB], alpha w_ep, alpha w_cost and zero, the
+// last look (FxLook), the
 // relaxed virtual controls, then the unextrapolated iterates of the stop test.
-struct FxLay { int vp, dx, gw, du, bq, th, ep, lo, hi, zx, kc, nvp, nvm, px, pu, pmp, pmm, pph, pth, end; };
+// The state at the last look (sn), a slot of `slot` entries for each lane, lies
+// in the FP64 loop's scratch, which is idle meanwhile, where it fits (6-DoF and
+// 3-DoF: always).
+struct FxLay {
+  int vp, dx, gw, du, bq, th, ep, lo, hi, zx, kc, lk, nvp, nvm, px, pu, pmp, pmm, pph, pth, sn, slot, end;
+};
 __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
   const int nup = KS_NC * ((L.nu + KS_NC - 1) / KS_NC), n1 = (L.N + 1) & ~1;
   FxLay Q;
@@ -180,6 +208,7 @@ __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
   Q.hi = o; o += n1 + 2;
   Q.zx = o; o += 2 * KS_NXB;
   Q.kc = o; o += 4;
+  Q.lk = o; o += 4;
   Q.nvp = o; o += L.N * KS_NXB;
   Q.nvm = o; o += L.N * KS_NXB;
   Q.px = o; o += L.N * KS_NXB;
@@ -189,17 +218,35 @@ __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
   Q.pph = o; o += L.N * KS_NXB;
   Q.pth = o; o += n1;
   Q.end = o;
+  Q.slot = KS_WC + 3 * KS_WR + nup / KS_NC + 1;
+  const int ns = L.N * KS_GS * Q.slot;
+  Q.sn = ns <= L.red - L.img ? L.img : Q.end;
+  if (Q.sn == Q.end) Q.end += ns;
   return Q;
 }
 
+// On fewer nodes the FP64 loop runs: the intervals of a reference that cannot be
+// flown on 4 or 5 nodes have blocks of up to 1e9, gamma falls below 1e-10, and
+// theta's increments round away (errors of 5e-13 and 7e-12 against 5e-14 and
+// 2e-14); large batches are no faster either (4096 solves at N = 2 to 5:
+// 0.8 to 1.1 of the FP64 loop's rate in the persistent form).
+constexpr int FX_NMIN = 6;
 // iterations between two looks at the magnitudes
 constexpr int FX_WINDOW = 10;
+// the last look: its iteration and unit, the iteration before which headroom is
+// kept, the parts run again so far, the coarsest unit (in shared memory: the
+// loop has no registers to spare)
+struct FxLook { int j, gb, hold, again, gtop; };
 
-// Returns the iterations run (at least one), or -1 with the image untouched;
-// *again the restarts at a coarser unit.
+// Returns the iterations run (at least one), or -1 with the image untouched.
+// Counts the parts run again at a coarser unit in P.loops[1].
 template <int NU>
-__device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, double sigma, int force, int* again) {
+__device__ __forceinline__ int phase_pipg_fx(const DParams& P, int nodes, double sigma, int force) {
   using U = unsigned long long;
+  if (nodes < FX_NMIN) return -1;
+  // the layout anew from the node count: offsets that the persistent kernel
+  // keeps in memory would be loaded once and then spilled around the loop
+  const Lay L = make_lay(nodes, NU, blockDim.x);
   extern __shared__ __align__(16) unsigned char smraw[];
   double* const sm = reinterpret_cast<double*>(smraw);
   constexpr int NXB = KS_NXB, TR = KS_TR, TC = KS_TC, NR = KS_NR, NCB = KS_NC, GS = KS_GS;
@@ -227,6 +274,7 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
   const double ga = alpha * so, gal = fma(alpha, so, -ga) + alpha * sol;
   // ---- scales, and whether the data suits (the same answer on every thread)
   U top[3] = {0, 0, 0};  // largest constant; largest iterate; largest |M|
+  unsigned cols = 0;     // control columns with an entry; with one of at least 2^-12
   {
     using OB = OrdBits<double>;
     for (int t = tid; t < (N - 1) * NX; t += blockDim.x) {
@@ -244,10 +292,13 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
     // (the padding entry of an odd block stride is not written)
     for (int t = tid; t < (N - 1) * NX * NU; t += blockDim.x) {
       const int k = t / (NX * NU), o = k * b_stride(NU) + t - k * (NX * NU);
-      top[2] = umax(top[2], umax(OB::abs(ga * sm[L.Bm + o]), OB::abs(ga * sm[L.Bp + o])));
+      const U b = umax(OB::abs(ga * sm[L.Bm + o]), OB::abs(ga * sm[L.Bp + o]));
+      top[2] = umax(top[2], b);
+      cols |= ((b > 0 ? 256u : 0u) | (b >= 0x3F30000000000000ull ? 1u : 0u)) << (t % NU);  // 2^-12
     }
     if (tid == 0) top[0] = umax(top[0], OB::abs(alpha * P.w_cost));
     block_max_u<U, 3>(top, reinterpret_cast<U*>(sm + L.red));
+    cols = block_or(cols, reinterpret_cast<unsigned*>(sm + L.red));
   }
   const double vc = __longlong_as_double((long long)top[0]), vs = __longlong_as_double((long long)top[1]);
   const double mx = __longlong_as_double((long long)top[2]);
@@ -260,7 +311,7 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
   // row's or column's sum of |M| stays below 5; an entry over 1.2 shows that
   // the power iteration fell short
   if (!(mx <= 1.2 && vc < 1e60 && vs < 1e60 && ref > 1e-60 && ga > 0.0 && ga <= 1.2 && P.rho > 0.0 && P.rho < 1.99 &&
-        alpha * wp < 1.0 && P.w_ep >= 0.0 && P.w_ep < 1e60))
+        alpha * wp < 1.0 && P.w_ep >= 0.0 && P.w_ep < 1e60 && (((cols >> 8) & ~cols & 255u) == 0 || ga < 0x1p-24)))
     return -1;
   const int gmin = ilogb(fmax(vc, 1e-60)) + 2;  // unit bound: constants below half of the range
   const FxC GM = fx_const(fx_prod(ga, gal, 1.0, 0x1p60));
@@ -320,8 +371,19 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
   const int jmax = force > 0 ? force : P.pipg_jmax;
   const bool chk_on = force <= 0 && P.pipg_jcheck > 0;
   const int per = chk_on ? P.pipg_jcheck : jmax;
-  int gb = ilogb(ref) + 3;  // range 8 to 16 times the largest quantity in sight
-  for (int attempt = 0; attempt < 4; ++attempt, gb += 6) {
+  // A part that leaves the range is run again from the last look's state.  With
+  // a stop test in every iteration that would need the unextrapolated iterates
+  // of the look as well; such a loop starts anew, and keeps its unit.
+  const bool roll = per > 1;
+  // range 4 to 8 times the largest quantity in sight; from a cold start, whose
+  // iterates grow for some hundred iterations, 16 to 32 times and with a bit of
+  // headroom kept that long (without: six parts run again, 3 % of 2000 iterations)
+  const bool cold = vs == 0.0;
+  int gb = ilogb(ref) + (cold ? 4 : 2);
+  FxLook* const look = reinterpret_cast<FxLook*>(ex + Q.lk);
+  if (tid == 0) *look = FxLook{0, gb, cold ? 300 : 0, 0, gb + 40};  // past gtop the iteration diverges
+  __syncthreads();
+  for (; gb <= look->gtop; gb += 2) {
     if (gb < gmin) gb = gmin;
     double sc = ldexp(1.0, 61 - gb);
     long long xt[WC], ft[WR], ut[NC], tht = 0;
@@ -384,7 +446,8 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         if (th_lane) ex[Q.th + g] = fx_mul(tht, GM);
       }
     };
-    for (int t = tid; t < Q.end - Q.vp; t += blockDim.x) ex[Q.vp + t] = 0;
+    for (int t = Q.vp + tid; t < Q.pth + N; t += blockDim.x)
+      if (t < Q.lk || t >= Q.nvp) ex[t] = 0;
     __syncthreads();
     constants();
 #pragma unroll
@@ -427,6 +490,47 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         any = any || (okd[e] && (ex[Q.nvp + g * NXB + i0 + e] | ex[Q.nvm + g * NXB + i0 + e]) != 0);
       nz = __any_sync(0xffffffffu, any);
     }
+    // the state at a look, in the unit of then
+    int j = 0;
+    long long* const slot = ex + Q.sn + (live ? tid : 0) * Q.slot;
+    auto save = [&]() {
+      if (live) {
+        long long* p = slot;
+#pragma unroll
+        for (int e = 0; e < WC; ++e) *p++ = xt[e];
+#pragma unroll
+        for (int e = 0; e < WR; ++e) {
+          *p++ = ft[e];
+          *p++ = ex[Q.nvp + g * NXB + i0 + e];
+          *p++ = ex[Q.nvm + g * NXB + i0 + e];
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) *p++ = ut[q];
+        *p = tht;
+      }
+      if (tid == 0) { look->j = j; look->gb = gb; }
+    };
+    auto restore = [&](int s) {  // at a unit 2^s times that of the look
+      bool any = false;
+      if (live) {
+        const long long* p = slot;
+#pragma unroll
+        for (int e = 0; e < WC; ++e) xt[e] = fx_shift(*p++, s);
+#pragma unroll
+        for (int e = 0; e < WR; ++e) {
+          ft[e] = fx_shift(*p++, s);
+          const long long a = fx_shift(*p++, s), b = fx_shift(*p++, s);
+          ex[Q.nvp + g * NXB + i0 + e] = a;
+          ex[Q.nvm + g * NXB + i0 + e] = b;
+          any = any || (a | b) != 0;
+        }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) ut[q] = fx_shift(*p++, s);
+        tht = fx_shift(*p, s);
+      }
+      if (wlive) nz = __any_sync(0xffffffffu, any);
+    };
+    if (roll) save();
     // V as in phase_pipg_ks: 0 plain, 1 stores the unextrapolated iterates,
     // 2 tests against the stored ones, then stores
     auto iterate = [&](auto v_tag) -> bool {
@@ -629,51 +733,77 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, const Lay& L, dou
         return false;
       }
     };
-    int j = 0;
     bool over = false;
-    while (j < jmax && !over) {
+    while (j < jmax) {
       // up to the next stop test, the next look at the magnitudes or the end
       // of the loop.  The last iteration before any of them stores the
-      // iterates that a test right behind it compares with.
-      const int to_test = per - j % per, to_look = FX_WINDOW - j % FX_WINDOW;
+      // iterates that a test right behind it compares with; where that test
+      // would be a part of its own, it closes this one.
+      const int to_test = per - j % per, to_look = FX_WINDOW - (j % per) % FX_WINDOW;
       int nb = to_test < jmax - j ? to_test : jmax - j;
       nb = to_look < nb ? to_look : nb;
+      if (to_test == nb + 1 && nb < jmax - j) nb = to_test;
       const bool tested = chk_on && nb == to_test;
       bool stop = false;
       for (int k = tested ? 2 : 1; k < nb; ++k) iterate(KsTag<0>{});
       if (!tested || nb >= 2) iterate(KsTag<1>{});
       if (tested) stop = iterate(KsTag<2>{});
-      j += nb;
       const unsigned m = block_or(mag, reinterpret_cast<unsigned*>(sm + L.red));
       mag = 0;
-      over = m >= (1u << 29);
-      if (stop || over || j >= jmax) break;
-      // keep one or two bits of headroom (no finer unit in the first
-      // iterations, whose iterates still grow)
-      const int slack = __clz(m) - 3;
-      int s = slack < 1 ? 2 - slack : (slack > 2 && j >= 3 * FX_WINDOW ? 1 - slack : 0);
-      if (gb + s < gmin) s = gmin - gb;
-      if (s != 0) {
-        gb += s;
-        sc = ldexp(1.0, 61 - gb);
+      if (m >= (1u << 29)) {
+        if (tid == 0) atomicAdd(P.loops + 1, 1ull);
+        over = !roll;
+        if (over) break;
+        gb += 2;
+        if (gb > look->gtop) return -1;
+        restore(gb - look->gb);
+        j = look->j;
+        if (tid == 0) {
+          look->again = look->again < 6 ? look->again + 1 : 6;
+          look->hold = j + (FX_WINDOW << look->again);
+        }
+      } else {
+        j += nb;
+        if (stop || j >= jmax) break;
+        // the largest magnitude to the top of the range, or (before hold) to
+        // one or two bits below it
+        const int slack = __clz(m) - 3;
+        int s = slack < 1 ? 2 : (roll && slack > 2 ? 1 - slack : 0);
+        if (roll && j >= look->hold) s = -slack;
+        if (gb + s < gmin) s = gmin - gb;
+        if (s != 0) {
+          gb += s;
 #pragma unroll
-        for (int e = 0; e < WC; ++e) xt[e] = fx_shift(xt[e], s);
+          for (int e = 0; e < WC; ++e) xt[e] = fx_shift(xt[e], s);
 #pragma unroll
-        for (int e = 0; e < WR; ++e) ft[e] = fx_shift(ft[e], s);
+          for (int e = 0; e < WR; ++e) ft[e] = fx_shift(ft[e], s);
 #pragma unroll
-        for (int q = 0; q < NC; ++q) ut[q] = fx_shift(ut[q], s);
-        tht = fx_shift(tht, s);
-        pm = umax(fx_mag(ft[0]), fx_mag(ft[1]));
-        for (int t = Q.nvp + tid; t < Q.end; t += blockDim.x) ex[t] = fx_shift(ex[t], s);
-        constants();
-        publish();
-        __syncthreads();
+          for (int q = 0; q < NC; ++q) ut[q] = fx_shift(ut[q], s);
+          tht = fx_shift(tht, s);
+          for (int t = Q.nvp + tid; t < Q.pth + N; t += blockDim.x) ex[t] = fx_shift(ex[t], s);
+        }
+        if (s == 0) {
+          if (roll) save();
+          continue;
+        }
       }
+      sc = ldexp(1.0, 61 - gb);
+      pm = umax(fx_mag(ft[0]), fx_mag(ft[1]));
+      constants();
+      publish();
+      __syncthreads();
+      if (roll) save();
     }
-    if (over) {
-      ++*again;
-      continue;
-    }
+    if (over) continue;
+    // whether every group of results keeps the precision that the FP64 loop's
+    // own exponents would give it (see the header)
+    U low[3] = {0, 0, 0};
+    for (int t = tid; t < N * NUP; t += blockDim.x) low[0] = umax(low[0], fx_abs(ex[Q.pu + t]));
+    for (int t = tid; t < (N - 1) * NXB; t += blockDim.x) low[1] = umax(low[1], fx_abs(ex[Q.pph + t]));
+    for (int t = tid; t < N - 1; t += blockDim.x) low[2] = umax(low[2], fx_abs(ex[Q.pth + t]));
+    block_max_u<U, 3>(low, reinterpret_cast<U*>(sm + L.red));
+    if (low[0] < (1ull << 53) || low[1] < (1ull << 53)) return -1;
+    if (low[2] != 0 && (low[2] < (1ull << 41) || P.eps_ctcs * P.Pxinv[IY] < ldexp(1.0, gb - 20))) return -1;
     // the unextrapolated iterates to the image (warm start of the next SCP iteration)
     const double un = ldexp(1.0, gb - 61);
     __syncthreads();

@@ -36,10 +36,10 @@ def test_steps_run_in_fixed_point(torch_cuda, oracle, inputs, model, nu):
     assert S.pipg_loops() == dict(fixed_point=0, again=0, fp64=0)
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 60))
     r = S.pipg_loops()
-    assert r["fixed_point"] == len(Ns) and r["fp64"] == 0
+    assert r["fixed_point"] == 6 and r["fp64"] == 2  # grids of fewer than 6 nodes run in FP64
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 3), phi=1e70)  # no unit suits
     r = S.pipg_loops()
-    assert r["fixed_point"] == len(Ns) and r["fp64"] == len(Ns)
+    assert r["fixed_point"] == 6 and r["fp64"] == 2 + len(Ns)
     S.set_threads(512)  # outside the fixed-point loop's thread counts
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 60))
     assert S.pipg_loops() == r
