@@ -20,7 +20,14 @@ namespace pdg {
 //
 // Products.  M is held as h 2^30 + l in units of 2^-60 (both signed, 32 bits),
 // an iterate is split as h 2^31 + 2 l; h h, h l and l h are summed in two
-// 64-bit accumulators, and l l (below half of the last unit) is left out.
+// 64-bit accumulators, and l l (below half of the last unit) is left out.  Of
+// the sum of h h and of the result only the low 64 bits count, so they may wrap
+// on the way.  The cross products must not: with |X| < 2^61 their sum is below
+// (s + n) 2^59 for n terms and a sum s of |M| over them, n <= 10 here, and the
+// loop is not entered with an s above FX_LANE.  Nor is it where the |M| of a
+// whole row or column, with the scalar terms beside it, come to more than
+// FX_SUM: then a result is below 7 2^61, and one that leaves the range cannot
+// wrap back into it unseen (default parameters: sums of 2.8 to 3.1).
 //
 // Range.  Every iterate that is multiplied or stored is or-ed into a word of
 // magnitudes; every 10 iterations the CTA looks at it.  The unit follows the
@@ -225,6 +232,14 @@ __host__ __device__ inline FxLay make_fx_lay(const Lay& L) {
   return Q;
 }
 
+// bounds on sums of |M|: over a lane's terms, over a whole row or column
+constexpr double FX_LANE = 5.5, FX_SUM = 6.0;
+// terms of a lane's longest sum: a tile column with x~ and the -I block, a tile
+// row with the controls of both nodes and the -I block
+__host__ __device__ constexpr int fx_terms(int nu) {
+  const int nc = (nu + KS_NC - 1) / KS_NC, row = KS_TC + 2 * nc + 1;
+  return KS_TR + 2 > row ? KS_TR + 2 : row;
+}
 // On fewer nodes the FP64 loop runs: the intervals of a reference that cannot be
 // flown on 4 or 5 nodes have blocks of up to 1e9, gamma falls below 1e-10, and
 // theta's increments round away (errors of 5e-13 and 7e-12 against 5e-14 and
@@ -307,9 +322,8 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, int nodes, double
   // it, x_hat after 20 iterations was off by 3.4e-11 at w_ep = 1e6 and 0.36 at
   // 1e16, relative to its largest; without it by 3e-16).
   const double ref = fmax(vc, vs);
-  // the range test of |M|: sigma bounds its spectral norm by one, so that a
-  // row's or column's sum of |M| stays below 5; an entry over 1.2 shows that
-  // the power iteration fell short
+  // the range test of |M|: sigma bounds its spectral norm by one; an entry over
+  // 1.2 shows that the power iteration fell short
   if (!(mx <= 1.2 && vc < 1e60 && vs < 1e60 && ref > 1e-60 && ga > 0.0 && ga <= 1.2 && P.rho > 0.0 && P.rho < 1.99 &&
         alpha * wp < 1.0 && P.w_ep >= 0.0 && P.w_ep < 1e60 && (((cols >> 8) & ~cols & 255u) == 0 || ga < 0x1p-24)))
     return -1;
@@ -352,6 +366,47 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, int nodes, double
   const long long c1 = (1LL << 60) - fx_prod(alpha, 0.0, wp, 0x1p60), g1 = fx_prod(ga, gal, 1.0, 0x1p60);
   const FxM cx1 = fx_entry(live ? c1 : 0), cu1 = fx_entry(live && rb == 0 ? c1 : 0);
   const FxM gxm = fx_entry(live ? -g1 : 0), gdm = fx_entry(has_iv ? -g1 : 0);
+  {  // the sums of |M|, in units of 2^-26 and rounded up
+    static_assert(FX_LANE + fx_terms(NU) < 16.0, "the cross products' accumulator");
+    auto mag = [](FxM m) { return (unsigned(m.h < 0 ? -m.h : m.h) >> 4) + 1u; };
+    const unsigned gm = mag(fx_entry(g1)), cm = mag(fx_entry(c1));
+    unsigned sum[4] = {0, 0, 0, 0};  // of a lane; rows and x columns; control columns of hat B^- and hat B^+
+    if (wlive) {
+      unsigned row[TR], rs[WR], col[TC], cs[WC];
+#pragma unroll
+      for (int q = 0; q < TC; ++q) col[q] = 0;
+#pragma unroll
+      for (int s = 0; s < TR; ++s) {
+        row[s] = 0;
+#pragma unroll
+        for (int q = 0; q < TC; ++q) { row[s] += mag(ap[s][q]); col[q] += mag(ap[s][q]); }
+#pragma unroll
+        for (int q = 0; q < NC; ++q) row[s] += mag(bm[s][q]) + mag(bp[s][q]);
+        sum[0] = umax(sum[0], row[s] + gm);
+      }
+#pragma unroll
+      for (int q = 0; q < TC; ++q) sum[0] = umax(sum[0], col[q] + cm + gm);
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        unsigned m = 0, p = 0;
+#pragma unroll
+        for (int s = 0; s < TR; ++s) { m += mag(bm[s][q]); p += mag(bp[s][q]); }
+        sum[0] = umax(sum[0], umax(m + cm, p));
+        sum[2] = umax(sum[2], ks_all_sum<NR, NCB>(m));
+        sum[3] = umax(sum[3], ks_all_sum<NR, NCB>(p));
+      }
+      ks_reduce_scatter<NCB, 1>(row, rs);
+      ks_reduce_scatter<NR, NCB>(col, cs);
+      // (theta enters a column twice, the constants up to half of the range)
+#pragma unroll
+      for (int e = 0; e < WR; ++e) sum[1] = umax(sum[1], rs[e] + gm);
+#pragma unroll
+      for (int e = 0; e < WC; ++e) sum[1] = umax(sum[1], cs[e] + cm + 3 * gm + (1u << 25));
+    }
+    block_max_u<unsigned, 4>(sum, reinterpret_cast<unsigned*>(sm + L.red));
+    constexpr unsigned top_sum = unsigned(FX_SUM * 0x1p26);
+    if (sum[0] > unsigned(FX_LANE * 0x1p26) || sum[1] > top_sum || sum[2] + sum[3] + cm > top_sum) return -1;
+  }
   bool fx[WC];
 #pragma unroll
   for (int e = 0; e < WC; ++e) {

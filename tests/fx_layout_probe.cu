@@ -90,7 +90,21 @@ static void check_disc(int N, int nu) {
 }
 #endif
 
+// The bound on the cross products' 64-bit sum: n terms |m.h| |v.l| + |m.l| |v.h|
+// with |v.l| and |m.l| <= 2^29, |v.h| <= 2^30, sum of |m.h| <= FX_LANE 2^30; and
+// on a result that left the range: it must not wrap to within 2^61 of zero.
+static void check_sums(int nu) {
+  ++cases;
+  const double cross = FX_LANE * 0x1p30 * 0x1p29 + fx_terms(nu) * 0x1p29 * 0x1p30 + 0x1p28;
+  CHECK(cross < 0x1p63, "nu=%d", nu);
+  // a dual row adds gamma w (half of the range) and the virtual controls (three eighths of it, times gamma <= 1.2)
+  CHECK(FX_SUM * 0x1p61 + 0x1p60 + 1.2 * 3 * 0x1p58 <= 0x1p64 - 0x1p61, "nu=%d", nu);
+  CHECK(KS_TR + 2 <= fx_terms(nu) && KS_TC + 2 * ((nu + KS_NC - 1) / KS_NC) + 1 <= fx_terms(nu), "nu=%d", nu);
+}
+
 int main() {
+  check_sums(4);
+  check_sums(PDG_MODEL_NU_ALT);
   const int nus[2] = {4, PDG_MODEL_NU_ALT};
   for (int a = 0; a < 2 && !(a == 1 && nus[1] == 4); ++a)
     for (int N = 2; N <= NMAX; ++N) {
