@@ -261,6 +261,14 @@ __host__ __device__ constexpr unsigned col_rows(int c) {
   return m;
 }
 
+// The barrier of the wave's stages.  The roles are branches of their own, and
+// __syncthreads() may stand in a branch only if all of the block take it; a
+// named barrier with its number of threads joins warps wherever they are (0.3 %
+// of the FP32 SCP iteration, 16384 instances, N = 15; nothing in FP64).
+__device__ __forceinline__ void disc_sync() {
+  asm volatile("barrier.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+}
+
 // RK4 state of one STM column: base, stage input, accumulator (entries outside
 // its rows are never used)
 template <typename R>
@@ -288,18 +296,18 @@ __device__ __forceinline__ void col_wave(ColState<R>& C, int c, const R* st, int
   const R h2 = R(0.5) * h, h6 = h / R(6);
 #pragma unroll
   for (int i = 0; i < NX; ++i) C.P[i] = C.S[i] = (i == c) ? R(1) : R(0);
-  __syncthreads();
+  disc_sync();
 #pragma unroll 1
   for (int n = 0; n < nsub; ++n) {
     const R l0 = R(n) / R(nsub), l1 = (R(n) + R(0.5)) / R(nsub), l2 = R(n + 1) / R(nsub);
     if (active) col_stage<R, NU, 0, ROWS, ACT, INH>(C, st, h, h2, h6, minus ? R(1) - l0 : l0, cu);
-    __syncthreads();
+    disc_sync();
     if (active) col_stage<R, NU, 1, ROWS, ACT, INH>(C, st + JS, h, h2, h6, minus ? R(1) - l1 : l1, cu);
-    __syncthreads();
+    disc_sync();
     if (active) col_stage<R, NU, 2, ROWS, ACT, INH>(C, st, h, h2, h6, minus ? R(1) - l1 : l1, cu);
-    __syncthreads();
+    disc_sync();
     if (active) col_stage<R, NU, 3, ROWS, ACT, INH>(C, st + JS, h, h2, h6, minus ? R(1) - l2 : l2, cu);
-    __syncthreads();
+    disc_sync();
   }
 }
 
@@ -398,11 +406,11 @@ __device__ __forceinline__ R discretize_cols(const DParams& P, const Lay& L, R* 
           for (int c = 0; c < NU - 1; ++c) J[SA_A + i * NU + c] = Bd[i * NU + c];
       };
       if (active) jac(0);
-      __syncthreads();
+      disc_sync();
 #pragma unroll 1
       for (int s = 0; s < S; ++s) {
         if (active && s + 1 < S) jac(s + 1);
-        __syncthreads();
+        disc_sync();
       }
     } else if (role.kind == 'F') {  // x, and of the Jacobians the CTCS row and the dilation's column
       const int k = k0 + lane;
@@ -442,11 +450,11 @@ __device__ __forceinline__ R discretize_cols(const DParams& P, const Lay& L, R* 
         for (int i = 0; i < NX; ++i) xP[i] = Xb[k * NX + i];
         x_stage(0);
       }
-      __syncthreads();
+      disc_sync();
 #pragma unroll 1
       for (int s = 0; s < S; ++s) {
         if (active && s + 1 < S) x_stage(s + 1);
-        __syncthreads();
+        disc_sync();
       }
       if (active) {
 #pragma unroll
@@ -465,17 +473,17 @@ __device__ __forceinline__ R discretize_cols(const DParams& P, const Lay& L, R* 
       for (int c = 0; c < COL_SINGLES; ++c)
 #pragma unroll
         for (int i = 0; i < NX; ++i) C[c].P[i] = C[c].S[i] = (i == c) ? R(1) : R(0);
-      __syncthreads();
+      disc_sync();
 #pragma unroll 1
       for (int n = 0; n < nsub; ++n) {
         if (active) singles_stage<R, NU, 0, 0>(C, st, h, h2, h6);
-        __syncthreads();
+        disc_sync();
         if (active) singles_stage<R, NU, 1, 0>(C, st + JS, h, h2, h6);
-        __syncthreads();
+        disc_sync();
         if (active) singles_stage<R, NU, 2, 0>(C, st, h, h2, h6);
-        __syncthreads();
+        disc_sync();
         if (active) singles_stage<R, NU, 3, 0>(C, st + JS, h, h2, h6);
-        __syncthreads();
+        disc_sync();
       }
       if (active) {
         singles_store<R, NU, 0>(P, L, sm, k, C);
@@ -497,7 +505,7 @@ __device__ __forceinline__ R discretize_cols(const DParams& P, const Lay& L, R* 
         for (int i = 0; i < NX; ++i) Bt[i * NU] = C.P[i] * pc * R(P.Pxinv[i]);
       }
     } else if (role.kind != 'C' || !classes_wave<R, NU, 0>(P, L, sm, D, role.index, W, k0, h)) {  // no columns
-      for (int s = 0; s < 4 * nsub + 1; ++s) __syncthreads();
+      for (int s = 0; s < 4 * nsub + 1; ++s) disc_sync();
     }
     __syncthreads();  // the next wave overwrites the stage buffers
   }
