@@ -230,7 +230,10 @@ int pdg_mc_launch_info(pdg_handle* h, int* threads, int* ctas_per_sm, int* smem_
 /* Override the threads-per-CTA of the solve kernels (multiple of 32 up to
  * 576, 0 = automatic).  Used by the autotuner.  PIPG forms 1 and 3 run at
  * most 512; forms 2 and 3 need a minimum (see pdg_mc_set_pipg_form); a solve
- * whose setting does not fit returns PDG_EINVAL. */
+ * whose setting does not fit returns PDG_EINVAL.  In FP64 form 1 the setting
+ * also decides between the fixed-point and the FP64 loop (there); within the
+ * former's range the plain form's PIPG and discretization kernels have their
+ * own sizes. */
 int pdg_mc_set_threads(pdg_handle* h, int threads);
 
 /* Autotune the launch shape for this handle's n_max, nu and precision on a

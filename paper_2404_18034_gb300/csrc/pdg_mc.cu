@@ -1066,7 +1066,7 @@ static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* 
     *out = {T, T < 128 ? 128 : T, 3, T, 3, 3};
   } else {
     // FP64 runs the loop in 64-bit fixed point (phase_pipg_fx: about three times
-    // the FP64 loop's rate: 2330 against 6890 cycles an instance and iteration
+    // the FP64 loop's rate: 2420 against 6890 cycles an instance and iteration
     // at N = 15) wherever its lane groups and its exchange region fit; not on
     // fewer than FX_NMIN nodes (see there), not with the thrust projection, whose
     // square roots are FP64 work, nor in a gradient's solve that records FP64

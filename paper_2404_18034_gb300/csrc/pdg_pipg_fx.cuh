@@ -68,11 +68,11 @@ namespace pdg {
 // Work split: the tiles and butterflies of phase_pipg_ks.  At N = 15 a CTA
 // runs 128 threads and about 4200 warp instructions an iteration, 900 of them
 // multiply-adds, against 382 FP64 instructions of 16 cycles each.  Measured
-// (4096 instances, N = 15): 30.1 ms per 1000 iterations, 2330 cycles an
+// (4096 instances, N = 15): 31.6 ms per 1000 iterations, 2420 cycles an
 // instance and iteration against 6890 of phase_pipg; N = 30 (1024 instances)
-// 15.9 ms.  Bound by latency and issue: two CTAs (8 warps) an SM at 255
-// registers, 1.4 instructions a clock; a third CTA at 168 registers adds
-// spills and no speed.
+// 16.0 ms; one instance alone 1.76 us an iteration (N = 10).  Bound by latency
+// and issue: two CTAs (8 warps) an SM at 255 registers, 1.4 instructions a
+// clock; a third CTA at 168 registers adds spills and no speed.
 // ---------------------------------------------------------------------------
 struct FxM { int h, l; };  // matrix entry: (h 2^30 + l) 2^-60
 struct FxC { int h, l2; };  // constant: (h 2^30 + l2 / 2) 2^-60
