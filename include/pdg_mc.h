@@ -257,9 +257,10 @@ int pdg_mc_autotune(pdg_handle* h, int B, const double* x0, const int* n_nodes, 
  *           thread count (one thread per block row or column, looped).  In
  *           FP64 the loop runs in 64-bit fixed point on form 3's lane groups
  *           where the thread count lies in [round32(8 N), 256] (4 N when
- *           NX <= 8), N >= 6, soc_thrust is off and the data suits, with
- *           errors no larger than the FP64 loop's; in FP64 otherwise (so that a
- *           thread setting outside that range, e.g. 288, asks for the FP64 loop);
+ *           NX <= 8), n_max >= 6 (in whole solves), soc_thrust is off and the
+ *           data suits, with errors no larger than the FP64 loop's; in FP64
+ *           otherwise (so that a thread setting outside that range, e.g. 288,
+ *           asks for the FP64 loop);
  *   form 2: every thread keeps its block rows/columns and iterate entries in
  *           registers for the whole loop; only the vectors exchanged between
  *           the primal and dual steps go through shared memory.  Needs

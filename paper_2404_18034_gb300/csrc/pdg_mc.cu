@@ -1037,8 +1037,10 @@ static size_t solve_smem(int N, int nu, int T, int kv) {
   return (size_t)(kv >= 4 ? make_fx_lay(L).end : L.total) * sizeof(R);
 }
 
-// B: instances of the launch (variant 6 is for batches of more than one an SM)
-static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* why, bool use_override = true) {
+// B: instances of the launch (variant 6 is for batches of more than one an SM);
+// step: a single SCP iteration
+static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* why, bool use_override = true,
+                     bool step = false) {
   const int treg = pipg_reg_threads(N, h->p.nu);
   const int maxt = h->p.precision == 1 ? PDG_REG_MAXT_F32 : 512;
   const int ov = use_override ? h->threads_override : 0;
@@ -1067,13 +1069,13 @@ static bool plan_for(const pdg_handle* h, int B, int N, Plan* out, std::string* 
   } else {
     // FP64 runs the loop in 64-bit fixed point (phase_pipg_fx: about three times
     // the FP64 loop's rate: 2420 against 6890 cycles an instance and iteration
-    // at N = 15) wherever its lane groups and its exchange region fit; not on
-    // fewer than FX_NMIN nodes (see there), not with the thrust projection, whose
-    // square roots are FP64 work, nor in a gradient's solve that records FP64
-    // states
+    // at N = 15) wherever its lane groups and its exchange region fit; not in
+    // whole solves on fewer than FX_NMIN nodes (see there), not with the thrust
+    // projection, whose square roots are FP64 work, nor in a gradient's solve that
+    // records FP64 states
     int T = ov > 0 ? ov : threads_for(N, h->p.nu, h->p.precision);
     if (T > 512) { *why = "the shared-memory PIPG form runs at most 512 threads per CTA"; return false; }
-    bool fx = h->p.precision == 0 && !h->p.soc_thrust && !h->ck_rec && N >= FX_NMIN;
+    bool fx = h->p.precision == 0 && !h->p.soc_thrust && !h->ck_rec && (step || N >= FX_NMIN);
     if (fx && ov == 0) T = T < tks ? tks : (T > PDG_FX_MAXT ? PDG_FX_MAXT : T);
     fx = fx && T >= tks && T <= PDG_FX_MAXT && solve_smem<double>(N, h->p.nu, T, 4) <= 226 * 1024;
     if (!fx && ov == 0) T = threads_for(N, h->p.nu, h->p.precision);
@@ -1363,7 +1365,7 @@ static int run_step(pdg_handle* h, int B, const double* x0, const int* Ns, doubl
                     double* step, int* iters, cudaStream_t s) {
   Plan pl;
   std::string why;
-  if (!plan_for(h, B, h->n_max, &pl, &why)) return fail(h, PDG_EINVAL, why);
+  if (!plan_for(h, B, h->n_max, &pl, &why, true, true)) return fail(h, PDG_EINVAL, why);
   const int T = pl.T, Tr = pl.Tr;
   const PlainPipgFn<R, NU> kpp = plain_pipg_fn<R, NU>(pl.kp);
   h->last_variant = pl.pv;

@@ -240,11 +240,13 @@ __host__ __device__ constexpr int fx_terms(int nu) {
   const int nc = (nu + KS_NC - 1) / KS_NC, row = KS_TC + 2 * nc + 1;
   return KS_TR + 2 > row ? KS_TR + 2 : row;
 }
-// On fewer nodes the FP64 loop runs: the intervals of a reference that cannot be
-// flown on 4 or 5 nodes have blocks of up to 1e9, gamma falls below 1e-10, and
-// theta's increments round away (errors of 5e-13 and 7e-12 against 5e-14 and
-// 2e-14); large batches are no faster either (4096 solves at N = 2 to 5:
-// 0.8 to 1.1 of the FP64 loop's rate in the persistent form).
+// On fewer nodes the FP64 loop runs where gamma is below 2^-7: the intervals of
+// a reference that cannot be flown on 4 or 5 nodes have blocks of up to 1e9,
+// gamma falls to 1e-10, and theta's increments round away (errors of 5e-13 and
+// 7e-12 against 5e-14 and 2e-14).  Nearly all SCP iterations but the first are
+// so there, and whole solves take the FP64 loop's kernels at once: large batches
+// are no faster in fixed point (4096 solves at N = 2 to 5, persistent form: 0.8 to
+// 1.1 of the FP64 loop's rate).
 constexpr int FX_NMIN = 6;
 // iterations between two looks at the magnitudes
 constexpr int FX_WINDOW = 10;
@@ -258,7 +260,6 @@ struct FxLook { int j, gb, hold, again, gtop; };
 template <int NU>
 __device__ __forceinline__ int phase_pipg_fx(const DParams& P, int nodes, double sigma, int force) {
   using U = unsigned long long;
-  if (nodes < FX_NMIN) return -1;
   // the layout anew from the node count: offsets that the persistent kernel
   // keeps in memory would be loaded once and then spilled around the loop
   const Lay L = make_lay(nodes, NU, blockDim.x);
@@ -325,7 +326,8 @@ __device__ __forceinline__ int phase_pipg_fx(const DParams& P, int nodes, double
   // the range test of |M|: sigma bounds its spectral norm by one; an entry over
   // 1.2 shows that the power iteration fell short
   if (!(mx <= 1.2 && vc < 1e60 && vs < 1e60 && ref > 1e-60 && ga > 0.0 && ga <= 1.2 && P.rho > 0.0 && P.rho < 1.99 &&
-        alpha * wp < 1.0 && P.w_ep >= 0.0 && P.w_ep < 1e60 && (((cols >> 8) & ~cols & 255u) == 0 || ga < 0x1p-24)))
+        alpha * wp < 1.0 && P.w_ep >= 0.0 && P.w_ep < 1e60 && (((cols >> 8) & ~cols & 255u) == 0 || ga < 0x1p-24) &&
+        (nodes >= FX_NMIN || ga >= 0x1p-7)))
     return -1;
   const int gmin = ilogb(fmax(vc, 1e-60)) + 2;  // unit bound: constants below half of the range
   const FxC GM = fx_const(fx_prod(ga, gal, 1.0, 0x1p60));

@@ -36,10 +36,10 @@ def test_steps_run_in_fixed_point(torch_cuda, oracle, inputs, model, nu):
     assert S.pipg_loops() == dict(fixed_point=0, again=0, fp64=0)
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 60))
     r = S.pipg_loops()
-    assert r["fixed_point"] == 6 and r["fp64"] == 2  # grids of fewer than 6 nodes run in FP64
+    assert r["fixed_point"] == len(Ns) and r["fp64"] == 0
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 3), phi=1e70)  # no unit suits
     r = S.pipg_loops()
-    assert r["fixed_point"] == 6 and r["fp64"] == 2 + len(Ns)
+    assert r["fixed_point"] == len(Ns) and r["fp64"] == len(Ns)
     S.set_threads(512)  # outside the fixed-point loop's thread counts
     _step(torch_cuda, S, p, oracle, x0, Ns, (20, 60))
     assert S.pipg_loops() == r
@@ -63,6 +63,11 @@ def test_solves_run_in_fixed_point(torch_cuda, inputs):
         want += 2 * B
         r = S.pipg_loops()
         assert r["fixed_point"] == want and r["fp64"] == 0
+    S.close()
+    S = Solver(p, 5)  # whole solves on fewer than six nodes: the FP64 loop's kernels
+    for mode in (0, 1):
+        S.solve(x0, mode=mode)
+    assert S.pipg_loops() == dict(fixed_point=0, again=0, fp64=0)
     S.close()
     for args in ((inputs.load_params(scp_jmax=2, pipg_jmax=100, soc_thrust=1), 0), (p, 1)):
         S = Solver(args[0], 12, args[1])  # the thrust projection; FP32
