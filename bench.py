@@ -36,11 +36,11 @@ METRIC = "converged PDG SCP solves/s on 1 GB300, batch 16384, N=15; % FP64/FP32 
 # kernel per instance, from ncu captures of the kernel sources with the given
 # hash (profiles/ has the summaries); reported only while the sources match.
 PROFILED_TRAFFIC = {
-    # ncu (dram__bytes_read.sum, dram__bytes_write.sum) of k_persistent<double,4,1> at
-    # its tuned 128 threads, 608 instances (one per CTA slot, four per SM):
-    # 6-DoF 14.10 MB read + 171.12 MB written; 3-DoF 3.107 MB read + 0.046 MB written
-    "40b1c3098dc7d69a": {("6dof", "fp64", 4, 15, "persistent"): 185.22e6 / 608,
-                         ("3dof", "fp64", 4, 15, "persistent"): 3.153e6 / 608},
+    # ncu (dram__bytes_read.sum, dram__bytes_write.sum) of k_persistent<double,4,5> at
+    # 128 threads, one instance per CTA slot: 6-DoF, 304 instances, 4.232 MB read +
+    # 1.081 MB written; 3-DoF, 456 instances, 4.595 MB read + 7.829 MB written
+    "40ecc0a32b326db7": {("6dof", "fp64", 4, 15, "persistent"): 5.313e6 / 304,
+                         ("3dof", "fp64", 4, 15, "persistent"): 12.424e6 / 456},
 }
 
 
